@@ -36,201 +36,308 @@ void cheb_weights(int p, double* w) {
   }
 }
 
-// All level kernels march along z: a block of 32 x 8 threads owns a 32 x 8
-// column of cells over ZC consecutive planes, each thread keeps the planes
-// below, at and above its cell in registers, and the in-plane neighbours come
-// through L1.  One DRAM read per input array per cell, with several planes'
-// loads in flight per thread.
-constexpr int ZC = 16;
+// One-cell kernels: the FP64 cycle, and the FP32 cycle on grids whose x-extent
+// is no multiple of 4.  A block of 32 x 8 threads owns a 32 x 8 column of
+// cells over zc consecutive planes; z-neighbours come from the registers of
+// the march, x-neighbours from the adjacent lanes by shuffles (loads at the
+// warp edges), y-neighbours through L1.
+//
+// GB300 issues FP64 arithmetic at two lanes per SM and clock (about 600 G
+// operations/s), so in FP64 the levels of 128^3 and above are bound by the
+// number of FP64 operations per cell, and the kernels are written to need few
+// of them: no division (1/nn from a table of selects), the six-neighbour sum
+// in four additions (the pair x(i-1,k) + x(i,k-1) serves the cells (i,k) and
+// (i-1,k-1)), the smoothing step in three operations on top of it, the
+// restriction from the differences across the faces of the coarse cell (the
+// differences inside it cancel; 4 operations per fine cell), the prolongation
+// separably with its powers of 1/4 in one factor (3 1/4).  Per V-cycle at the
+// finest level about 30 FP64 operations per cell.  Measured at 192^3 in FP64
+// (us per launch, in brackets one cell's plain sums and quotients in marches
+// of 16 planes): k_first 115 (513), k_sweep 112 (249; 94 at 600 G/s),
+// k_restrict 77 (133), k_prolong 61 (174), the V-cycle 612 (2230).
+// The levels below 64^3 are bound by latency: one plane per thread (zm_planes)
+// and programmatic dependent launch.
+//
+// Weights come from tables formed on the host and picked by selects, so that a
+// thread of few planes spends no FP64 operation on them.
+constexpr int kZcMax = 8;
 
-dim3 zm_grid(Dims d) { return dim3(div_up(d.nx, BX), div_up(d.ny, BY), div_up(d.nz, ZC)); }
+// planes per thread: about eight blocks per SM over the grid, at most 8 (six
+// blocks fit an SM: several waves keep its last one short)
+int zm_planes(Dims d) {
+  const int64_t bxy = (int64_t)div_up(d.nx, BX) * div_up(d.ny, BY);
+  return (int)std::min<int64_t>(kZcMax, std::max<int64_t>(1, d.nz * bxy / (152 * 8)));
+}
 
-// w / nn for nn = 0..6 (nn = number of existing neighbours of a cell).
+dim3 zm_grid(Dims d, int zc) {
+  return dim3(div_up(d.nx, BX), div_up(d.ny, BY), div_up(d.nz, zc));
+}
+
+// w / nn for the neighbour counts 3..6 (every axis of a level that is
+// smoothed has at least four cells)
 template <typename T>
-struct WOverN {
-  T v[7];
+struct OverCount {
+  T v3, v4, v5, v6;
 };
 
 template <typename T>
-WOverN<T> w_over_n(double w) {
-  WOverN<T> r;
-  r.v[0] = (T)0;
-  for (int q = 1; q < 7; ++q) r.v[q] = (T)(w / q);
-  return r;
+OverCount<T> over_count(double w) {
+  return {(T)(w / 3.0), (T)(w / 4.0), (T)(w / 5.0), (T)(w / 6.0)};
 }
 
-// w / nn from the table with static indices only (a dynamically indexed
-// kernel-parameter array would be copied to local memory): interior cells
-// (nn = 6) use the stored quotient, boundary cells divide.
 template <typename T>
-__device__ __forceinline__ T wn_of(const WOverN<T>& wn, int nn) {
-  return nn == 6 ? wn.v[6] : wn.v[1] / (T)nn;
+__device__ __forceinline__ T by_count(const OverCount<T>& w, int nn) {
+  return nn >= 6 ? w.v6 : (nn == 5 ? w.v5 : (nn == 4 ? w.v4 : w.v3));
+}
+
+// -nn without a conversion (which runs on the FP64 pipe)
+template <typename T>
+__device__ __forceinline__ T neg_count(int nn) {
+  return nn >= 6 ? (T)-6 : (nn == 5 ? (T)-5 : (nn == 4 ? (T)-4 : (T)-3));
+}
+
+// Weights of the first two steps away from the y and z walls (see k_first).
+template <typename T>
+struct FirstWeights {
+  T w0h2, w1, omw1, h2;    // w0 h^2, w1, 1 - w1, h^2
+  T k6, k5;                // own weight for six and for five neighbours
+  T p66, p65, p55;         // neighbour's weight by the two cells' counts
+  OverCount<T> inv, w0h2n, w1n;   // 1 / nn, w0 h^2 / nn, w1 / nn
+};
+
+template <typename T>
+FirstWeights<T> first_weights(double w0, double w1, double h2) {
+  auto k = [&](double n) { return (T)((1.0 - w1) * w0 * h2 / n + w1 / n * h2); };
+  auto p = [&](double n, double q) { return (T)(w1 / n * (w0 * h2 / q)); };
+  return {(T)(w0 * h2),       (T)w1,         (T)(1.0 - w1),  (T)h2,
+          k(6.0),             k(5.0),        p(6.0, 6.0),    p(6.0, 5.0),
+          p(5.0, 5.0),        over_count<T>(1.0), over_count<T>(w0 * h2), over_count<T>(w1)};
 }
 
 __device__ __forceinline__ int n_inplane(Dims d, int i, int j) {
   return (i > 0) + (i < d.nx - 1) + (j > 0) + (j < d.ny - 1);
 }
 
-template <typename T>
-__device__ __forceinline__ T inplane_sum(const T* __restrict__ p, int64_t c, int i, int j, Dims d,
-                                         int64_t sy) {
-  T s = 0;
-  if (i > 0) s += __ldg(p + c - 1);
-  if (i < d.nx - 1) s += __ldg(p + c + 1);
-  if (j > 0) s += __ldg(p + c - sy);
-  if (j < d.ny - 1) s += __ldg(p + c + sy);
-  return s;
-}
-
 // One Chebyshev-Richardson step: xo = x + w D^{-1} (b - L x), D = nn / h^2,
-// L x = (nn x_c - sum of neighbours) / h^2.  b may be FP64 while T is FP32,
-// and the output type TO may differ from T (FP64 result of the mixed cycle).
+// L x = (nn x_c - sum of neighbours) / h^2.
+// b may be FP64 while T is FP32, and the output type TO may differ from T
+// (FP64 result of the mixed cycle).
 template <typename T, typename TB, typename TO>
 __global__ void __launch_bounds__(BX * BY) k_sweep(Dims d, const T* __restrict__ x,
                                                    const TB* __restrict__ b, TO* __restrict__ xo,
-                                                   WOverN<T> wn, T h2) {
-  const int i = blockIdx.x * BX + threadIdx.x;
+                                                   const OverCount<T> w, T h2, int zc) {
+  pdl_wait();
+  pdl_trigger();
+  const int lane = threadIdx.x;
+  const int i = blockIdx.x * BX + lane;
   const int j = blockIdx.y * BY + threadIdx.y;
-  if (i >= d.nx || j >= d.ny) return;
-  const int z0 = blockIdx.z * ZC;
-  const int z1 = min(z0 + ZC, d.nz);
+  const bool act = i < d.nx && j < d.ny;
+  const int z0 = blockIdx.z * zc;
+  const int z1 = min(z0 + zc, d.nz);
   const int64_t sy = d.nx, sz = (int64_t)d.nx * d.ny;
   const int nip = n_inplane(d, i, j);
+  const T w_in = by_count(w, nip + 2), w_wall = by_count(w, nip + 1);
+  const T n_in = neg_count<T>(nip + 2), n_wall = neg_count<T>(nip + 1);
+  const bool hym = act && j > 0, hyp = act && j < d.ny - 1;
+  const bool edge_l = act && lane == 0 && i > 0, edge_r = act && lane == 31 && i < d.nx - 1;
   int64_t c = (int64_t)z0 * sz + (int64_t)j * sy + i;
-  T xp = z0 > 0 ? __ldg(x + c - sz) : (T)0;
-  T xc = __ldg(x + c);
-#pragma unroll 4
+  const T xp = (act && z0 > 0) ? __ldg(x + c - sz) : (T)0;
+  T xc = act ? __ldg(x + c) : (T)0;
+  T xl = __shfl_up_sync(0xffffffffu, xc, 1);
+  if (lane == 0) xl = edge_l ? __ldg(x + c - 1) : (T)0;
+  T dc = xl + xp;   // x(i-1, z) + x(i, z-1)
   for (int z = z0; z < z1; ++z, c += sz) {
-    const T xn = (z + 1 < d.nz) ? __ldg(x + c + sz) : (T)0;
-    const int nn = nip + (z > 0) + (z < d.nz - 1);
-    const T s = inplane_sum(x, c, i, j, d, sy) + (xp + xn);
-    const T r = fma(h2, (T)__ldg(b + c), s - (T)nn * xc);
-    xo[c] = (TO)fma(wn_of(wn, nn), r, xc);
-    xp = xc;
+    const bool up = z + 1 < d.nz;
+    const T xn = (act && up) ? __ldg(x + c + sz) : (T)0;
+    const T ym = hym ? __ldg(x + c - sy) : (T)0;
+    const T yp = hyp ? __ldg(x + c + sy) : (T)0;
+    const T bv = act ? (T)__ldg(b + c) : (T)0;
+    T xnl = __shfl_up_sync(0xffffffffu, xn, 1);
+    if (lane == 0) xnl = (edge_l && up) ? __ldg(x + c + sz - 1) : (T)0;
+    const T dn = xnl + xc;                            // x(i-1, z+1) + x(i, z)
+    T dr = __shfl_down_sync(0xffffffffu, dn, 1);      // x(i, z+1) + x(i+1, z)
+    if (lane == 31) dr = edge_r ? xn + __ldg(x + c + 1) : xn;
+    const T s = (dc + dr) + (ym + yp);
+    const bool in = z > 0 && up;
+    if (act) xo[c] = (TO)fma(in ? w_in : w_wall, fma(h2, bv, fma(in ? n_in : n_wall, xc, s)), xc);
+    dc = dn;
     xc = xn;
   }
 }
 
 // First smoothing step(s) from a zero iterate.  x1 = w0 D^{-1} b pointwise; with
 // two != 0 also the second step xo = x1 + w1 D^{-1} (b - L x1), evaluating x1 at
-// the neighbours from b on the fly (no x1 array).  bcopy (may be null) receives
-// b rounded to T, for the later kernels of the level.
+// the neighbours from b on the fly (no x1 array).  Two cells and more away
+// from every wall both steps are one stencil on b with three weights; along
+// the x-walls the two x-neighbours have weights of their own.  bcopy (may be
+// null) receives b rounded to T, for the later kernels of the level.
 template <typename T, typename TB>
 __global__ void __launch_bounds__(BX * BY) k_first(Dims d, const TB* __restrict__ b,
                                                    T* __restrict__ bcopy, T* __restrict__ xo,
-                                                   WOverN<T> w0h2n, WOverN<T> w1n, T h2, int two) {
-  const int i = blockIdx.x * BX + threadIdx.x;
+                                                   const FirstWeights<T> w, int two, int zc) {
+  pdl_wait();
+  pdl_trigger();
+  const int lane = threadIdx.x;
+  const int i = blockIdx.x * BX + lane;
   const int j = blockIdx.y * BY + threadIdx.y;
-  if (i >= d.nx || j >= d.ny) return;
-  const int z0 = blockIdx.z * ZC;
-  const int z1 = min(z0 + ZC, d.nz);
+  const bool act = i < d.nx && j < d.ny;
+  const int z0 = blockIdx.z * zc;
+  const int z1 = min(z0 + zc, d.nz);
   const int64_t sy = d.nx, sz = (int64_t)d.nx * d.ny;
   const int nip = n_inplane(d, i, j);
   int64_t c = (int64_t)z0 * sz + (int64_t)j * sy + i;
+  auto nzc = [&](int z) { return (z > 0) + (z < d.nz - 1); };
   if (!two) {
+    if (!act) return;
     for (int z = z0; z < z1; ++z, c += sz) {
       const T bv = (T)__ldg(b + c);
       if (bcopy) bcopy[c] = bv;
-      xo[c] = wn_of(w0h2n, nip + (z > 0) + (z < d.nz - 1)) * bv;
+      xo[c] = by_count(w.w0h2n, nip + nzc(z)) * bv;
     }
     return;
   }
-  // in-plane neighbour counts of the four in-plane neighbours
-  const int nxm = i > 0 ? n_inplane(d, i - 1, j) : 0;
-  const int nxp = i < d.nx - 1 ? n_inplane(d, i + 1, j) : 0;
-  const int nym = j > 0 ? n_inplane(d, i, j - 1) : 0;
-  const int nyp = j < d.ny - 1 ? n_inplane(d, i, j + 1) : 0;
-  auto nzc = [&](int z) { return (z > 0) + (z < d.nz - 1); };
-  // x1 below / at / above, carried along z
-  T x1p = z0 > 0 ? wn_of(w0h2n, nip + nzc(z0 - 1)) * (T)__ldg(b + c - sz) : (T)0;
-  T bcv = (T)__ldg(b + c);
-  T x1c = wn_of(w0h2n, nip + nzc(z0)) * bcv;
-#pragma unroll 2
+  // with x1 = r b, r = w0 h^2 / nn: x2 = c0 b + (w1/nn) sum_nb r_nb b_nb,
+  // c0 = (1 - w1) r + (w1/nn) h^2
+  const bool hxm = act && i > 0, hxp = act && i < d.nx - 1;
+  const bool hym = act && j > 0, hyp = act && j < d.ny - 1;
+  const bool yin = j >= 2 && j <= d.ny - 3;
+  // a warp two cells off the x-walls: one weight for all six neighbours, their
+  // sum in four additions (dc as in k_sweep)
+  const bool xin = blockIdx.x > 0 && (blockIdx.x + 1) * BX + 2 <= d.nx;
+  // five neighbours next to an x-wall, six elsewhere (off the y and z walls)
+  const bool o6 = i > 0 && i < d.nx - 1;
+  const T k0 = o6 ? w.k6 : w.k5, ky = o6 ? w.p66 : w.p55;
+  // an x-neighbour beyond the wall is read as 0, whatever its weight
+  const T kl = (o6 && i - 1 > 0) ? w.p66 : w.p65, kr = (o6 && i + 1 < d.nx - 1) ? w.p66 : w.p65;
+  const bool edge_l = hxm && lane == 0, edge_r = hxp && lane == 31;
+  T bp = (act && z0 > 0) ? (T)__ldg(b + c - sz) : (T)0;
+  T bc = act ? (T)__ldg(b + c) : (T)0;
+  T xl = __shfl_up_sync(0xffffffffu, bc, 1);
+  if (lane == 0) xl = edge_l ? (T)__ldg(b + c - 1) : (T)0;
+  T dc = xin ? xl + bp : (T)0;   // b(i-1, z) + b(i, z-1)
   for (int z = z0; z < z1; ++z, c += sz) {
-    T bnv = 0, x1n = 0;
-    if (z + 1 < d.nz) {
-      bnv = (T)__ldg(b + c + sz);
-      x1n = wn_of(w0h2n, nip + nzc(z + 1)) * bnv;
+    const bool up = z + 1 < d.nz;
+    const T bn = (act && up) ? (T)__ldg(b + c + sz) : (T)0;
+    const T ym = hym ? (T)__ldg(b + c - sy) : (T)0;
+    const T yp = hyp ? (T)__ldg(b + c + sy) : (T)0;
+    T bnl = __shfl_up_sync(0xffffffffu, bn, 1);
+    if (lane == 0) bnl = (edge_l && up) ? (T)__ldg(b + c + sz - 1) : (T)0;
+    T o;
+    const bool in = yin && z >= 2 && z <= d.nz - 3;   // warp-uniform, as xin
+    T s = 0, dn = 0;
+    if (xin) {
+      dn = bnl + bc;
+      T dr = __shfl_down_sync(0xffffffffu, dn, 1);
+      if (lane == 31) dr = bn + (act ? (T)__ldg(b + c + 1) : (T)0);   // off the walls
+      if (in) s = (dc + dr) + (ym + yp);
     }
-    const int zc = nzc(z);
-    T s = x1p + x1n;
-    if (i > 0) s += wn_of(w0h2n, nxm + zc) * (T)__ldg(b + c - 1);
-    if (i < d.nx - 1) s += wn_of(w0h2n, nxp + zc) * (T)__ldg(b + c + 1);
-    if (j > 0) s += wn_of(w0h2n, nym + zc) * (T)__ldg(b + c - sy);
-    if (j < d.ny - 1) s += wn_of(w0h2n, nyp + zc) * (T)__ldg(b + c + sy);
-    const int nn = nip + zc;
-    if (bcopy) bcopy[c] = bcv;
-    const T r = fma(h2, bcv, s - (T)nn * x1c);
-    xo[c] = fma(wn_of(w1n, nn), r, x1c);
-    x1p = x1c;
-    x1c = x1n;
-    bcv = bnv;
+    if (xin && in) {
+      o = fma(k0, bc, ky * s);
+    } else {
+      T xr = __shfl_down_sync(0xffffffffu, bc, 1);
+      if (lane == 31) xr = edge_r ? (T)__ldg(b + c + 1) : (T)0;
+      if (in) {
+        o = fma(k0, bc, fma(kl, xl, fma(kr, xr, ky * ((ym + yp) + (bp + bn)))));
+      } else {
+        // counts of the cell and its neighbours; absent ones hold b = 0
+        const int zn = nzc(z), nn = nip + zn;
+        const int nym = nn + (j - 1 > 0) - (j > 0) + 1 - (j < d.ny - 1);
+        const int nyp = nn + (j + 1 < d.ny - 1) - (j < d.ny - 1) + 1 - (j > 0);
+        const int nxm = nn + (i - 1 > 0) - (i > 0) + 1 - (i < d.nx - 1);
+        const int nxp = nn + (i + 1 < d.nx - 1) - (i < d.nx - 1) + 1 - (i > 0);
+        s = fma(by_count(w.inv, nn + nzc(z - 1) - zn), bp, by_count(w.inv, nn + nzc(z + 1) - zn) * bn) +
+            fma(by_count(w.inv, nym), ym, by_count(w.inv, nyp) * yp) +
+            fma(by_count(w.inv, nxm), xl, by_count(w.inv, nxp) * xr);
+        o = fma(by_count(w.w1n, nn), fma(w.w0h2, s, w.h2 * bc),
+                w.omw1 * (by_count(w.w0h2n, nn) * bc));
+      }
+    }
+    if (act) {
+      if (bcopy) bcopy[c] = bc;
+      xo[c] = o;
+    }
+    dc = dn;
+    bp = bc;
+    bc = bn;
+    xl = bnl;
   }
 }
 
 // Residual restriction: bcoarse = average over the 8 children of (b - L x);
-// x == nullptr means x = 0.  One thread per coarse cell; the children are read
-// in x-pairs (2I, 2I+1).
+// x == nullptr means x = 0.  A thread owns one fine x and the two fine rows of
+// a coarse one, and marches over the coarse planes.  The sum of L x over the
+// children is the sum of the differences across the coarse cell's faces.
 template <typename T>
-struct Pair;
-template <>
-struct Pair<float> {
-  using type = float2;
-};
-template <>
-struct Pair<double> {
-  using type = double2;
-};
-
-template <typename T>
-__device__ __forceinline__ void ld2(const T* p, T& a, T& b) {
-  const typename Pair<T>::type v = __ldg(reinterpret_cast<const typename Pair<T>::type*>(p));
-  a = v.x;
-  b = v.y;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(BX * BY) k_restrict(Dims d, Dims dc, const T* __restrict__ x,
+__global__ void __launch_bounds__(BX * BY, 4) k_restrict(Dims d, Dims dc, const T* __restrict__ x,
                                                       const T* __restrict__ b,
-                                                      T* __restrict__ bcoarse, T inv_h2) {
-  const int I = blockIdx.x * BX + threadIdx.x;
+                                                      T* __restrict__ bcoarse, T inv_h2, int zcc) {
+  pdl_wait();
+  pdl_trigger();
+  const int lane = threadIdx.x;
+  const int i = blockIdx.x * BX + lane;
   const int J = blockIdx.y * BY + threadIdx.y;
-  if (I >= dc.nx || J >= dc.ny) return;
+  const bool act = i < d.nx && J < dc.ny;   // nx is even: both cells of a pair are
   const int64_t sy = d.nx, sz = (int64_t)d.nx * d.ny;
-  const int K0 = blockIdx.z * (ZC / 2);
-  const int K1 = min(K0 + ZC / 2, dc.nz);
-  for (int K = K0; K < K1; ++K) {
-    T acc = 0;
-#pragma unroll
-    for (int dz = 0; dz < 2; ++dz) {
-      const int k = 2 * K + dz;
-#pragma unroll
-      for (int dy = 0; dy < 2; ++dy) {
-        const int j = 2 * J + dy;
-        const int64_t c = (int64_t)k * sz + (int64_t)j * sy + 2 * I;
-        T b0, b1;
-        ld2(b + c, b0, b1);
-        T r0 = b0, r1 = b1;
-        if (x) {
-          T x0, x1;
-          ld2(x + c, x0, x1);
-          // neighbours of the pair
-          T s0 = x1, s1 = x0;
-          int n0 = 1, n1 = 1;
-          if (2 * I > 0) { s0 += __ldg(x + c - 1); ++n0; }
-          if (2 * I + 2 < d.nx) { s1 += __ldg(x + c + 2); ++n1; }
-          T a0, a1;
-          if (j > 0) { ld2(x + c - sy, a0, a1); s0 += a0; s1 += a1; ++n0; ++n1; }
-          if (j < d.ny - 1) { ld2(x + c + sy, a0, a1); s0 += a0; s1 += a1; ++n0; ++n1; }
-          if (k > 0) { ld2(x + c - sz, a0, a1); s0 += a0; s1 += a1; ++n0; ++n1; }
-          if (k < d.nz - 1) { ld2(x + c + sz, a0, a1); s0 += a0; s1 += a1; ++n0; ++n1; }
-          r0 -= ((T)n0 * x0 - s0) * inv_h2;
-          r1 -= ((T)n1 * x1 - s1) * inv_h2;
+  const int K0 = blockIdx.z * zcc;
+  const int K1 = min(K0 + zcc, dc.nz);
+  const bool hym = act && J > 0, hyp = act && J < dc.ny - 1;
+  // the x-neighbour outside the pair: left of an even cell, right of an odd one
+  const bool wallx = (lane & 1) ? i == d.nx - 1 : i == 0;
+  const int src = (lane & 1) ? lane + 1 : lane - 1;
+  const bool edge = act && !wallx && (lane == 0 || lane == 31);
+  const int64_t eo = lane == 0 ? -1 : 1;
+  int64_t c = (int64_t)(2 * K0) * sz + (int64_t)(2 * J) * sy + i;
+  // sum of the two rows' x at the planes 2K-1, 2K, 2K+1, 2K+2
+  T sm = 0, s0 = 0, a0 = 0, a1 = 0;
+  if (x && act) {
+    a0 = __ldg(x + c);
+    a1 = __ldg(x + c + sy);
+    s0 = a0 + a1;
+    sm = K0 > 0 ? __ldg(x + c - sz) + __ldg(x + c - sz + sy) : s0;
+  }
+  for (int K = K0; K < K1; ++K, c += 2 * sz) {
+    T r = 0, t = 0;
+    if (act)
+      r = (__ldg(b + c) + __ldg(b + c + sy)) + (__ldg(b + c + sz) + __ldg(b + c + sz + sy));
+    if (x) {
+      T e0 = 0, e1 = 0, n0 = 0, n1 = 0;
+      T m0 = a0, m1 = 0, p0 = a1, p1 = 0;   // y-neighbours of the two planes
+      if (act) {
+        e0 = __ldg(x + c + sz);
+        e1 = __ldg(x + c + sz + sy);
+        m1 = e0;
+        p1 = e1;
+        if (K < dc.nz - 1) {
+          n0 = __ldg(x + c + 2 * sz);
+          n1 = __ldg(x + c + 2 * sz + sy);
         }
-        acc += r0 + r1;
+        if (hym) {
+          m0 = __ldg(x + c - sy);
+          m1 = __ldg(x + c + sz - sy);
+        }
+        if (hyp) {
+          p0 = __ldg(x + c + 2 * sy);
+          p1 = __ldg(x + c + sz + 2 * sy);
+        }
       }
+      const T s1 = e0 + e1, s2 = n0 + n1;
+      const T cc = s0 + s1;
+      T oc = __shfl_sync(0xffffffffu, cc, src & 31);
+      if (lane == 0 || lane == 31)
+        oc = edge ? (__ldg(x + c + eo) + __ldg(x + c + sy + eo)) +
+                        (__ldg(x + c + sz + eo) + __ldg(x + c + sz + sy + eo))
+                  : (T)0;
+      if (wallx) oc = cc;
+      t = fma((T)3, cc,
+              -((oc + ((m0 + p0) + (m1 + p1))) + (sm + (K < dc.nz - 1 ? s2 : s1))));
+      sm = s1;
+      s0 = s2;
+      a0 = n0;
+      a1 = n1;
     }
-    bcoarse[((int64_t)K * dc.ny + J) * dc.nx + I] = acc * (T)0.125;
+    r = fma(-inv_h2, t, r);
+    r += __shfl_xor_sync(0xffffffffu, r, 1);
+    if (act && !(lane & 1)) bcoarse[((int64_t)K * dc.ny + J) * dc.nx + (i >> 1)] = r * (T)0.125;
   }
 }
 
@@ -242,48 +349,60 @@ __global__ void k_convert(const T* __restrict__ x, TO* __restrict__ y, int64_t n
 }
 
 // x (+)= P xc: trilinear, 3/4 parent and 1/4 neighbour per axis, the
-// neighbour replaced by the parent at a wall.  One thread per fine x-pair
-// (2I, 2I+1), which share the parent I; overwrite != 0 gives x = P xc.
+// neighbour replaced by the parent at a wall; overwrite != 0 gives x = P xc.
+// A thread owns one fine x and the two fine rows of a coarse one, and marches
+// over the coarse planes: 3 a + b along x, then y, then z, times 1/64.
 template <typename T>
 __global__ void __launch_bounds__(BX * BY) k_prolong(Dims d, Dims dc, const T* __restrict__ xc,
-                                                     T* __restrict__ x, int overwrite) {
-  const int I = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  if (I >= dc.nx || j >= d.ny) return;
-  const int z0 = blockIdx.z * ZC;
-  const int z1 = min(z0 + ZC, d.nz);
-  const int J = j >> 1;
-  const int Jn = (j & 1) ? min(J + 1, dc.ny - 1) : max(J - 1, 0);
-  const int Im = max(I - 1, 0), Ip = min(I + 1, dc.nx - 1);
+                                                     T* __restrict__ x, int overwrite, int zcc) {
+  pdl_wait();
+  pdl_trigger();
+  const int i = blockIdx.x * BX + threadIdx.x;
+  const int J = blockIdx.y * BY + threadIdx.y;
+  if (i >= d.nx || J >= dc.ny) return;
+  const int K0 = blockIdx.z * zcc;
+  const int K1 = min(K0 + zcc, dc.nz);
+  const int I = i >> 1;
+  const int In = (i & 1) ? min(I + 1, dc.nx - 1) : max(I - 1, 0);
   const int64_t sy = dc.nx, sz = (int64_t)dc.nx * dc.ny;
-  for (int k = z0; k < z1; ++k) {
-    const int K = k >> 1;
-    const int Kn = (k & 1) ? min(K + 1, dc.nz - 1) : max(K - 1, 0);
-    // rows (J, K), (Jn, K), (J, Kn), (Jn, Kn); 3/4-1/4 in y and z first
-    const T* r00 = xc + K * sz + J * sy;
-    const T* r01 = xc + K * sz + Jn * sy;
-    const T* r10 = xc + Kn * sz + J * sy;
-    const T* r11 = xc + Kn * sz + Jn * sy;
-    auto yz = [&](int q) {
-      const T a = (T)0.75 * __ldg(r00 + q) + (T)0.25 * __ldg(r01 + q);
-      const T bb = (T)0.75 * __ldg(r10 + q) + (T)0.25 * __ldg(r11 + q);
-      return (T)0.75 * a + (T)0.25 * bb;
-    };
-    const T cm = yz(Im), c0 = yz(I), cp = yz(Ip);
-    const T v0 = (T)0.75 * c0 + (T)0.25 * cm;   // fine 2I   (neighbour I-1)
-    const T v1 = (T)0.75 * c0 + (T)0.25 * cp;   // fine 2I+1 (neighbour I+1)
-    const int64_t f = ((int64_t)k * d.ny + j) * d.nx + 2 * I;
-    typename Pair<T>::type* px = reinterpret_cast<typename Pair<T>::type*>(x + f);
-    typename Pair<T>::type o;
+  const int64_t rm = max(J - 1, 0) * sy, rc = J * sy, rp = min(J + 1, dc.ny - 1) * sy;
+  // the two fine rows on coarse plane K
+  auto rows = [&](int K, T& lo, T& hi) {
+    const T* p = xc + K * sz;
+    const T gm = fma((T)3, __ldg(p + rm + I), __ldg(p + rm + In));
+    const T gc = fma((T)3, __ldg(p + rc + I), __ldg(p + rc + In));
+    const T gp = fma((T)3, __ldg(p + rp + I), __ldg(p + rp + In));
+    lo = fma((T)3, gc, gm);
+    hi = fma((T)3, gc, gp);
+  };
+  T pl, ph, cl, ch;
+  rows(K0, cl, ch);
+  rows(max(K0 - 1, 0), pl, ph);
+  const int64_t fy = d.nx, fz = (int64_t)d.nx * d.ny;
+  int64_t f = (int64_t)(2 * K0) * fz + (int64_t)(2 * J) * fy + i;
+  const T q = (T)(1.0 / 64.0);
+  for (int K = K0; K < K1; ++K, f += 2 * fz) {
+    T nl, nh;
+    rows(min(K + 1, dc.nz - 1), nl, nh);
+    const T v0 = fma((T)3, cl, pl), v1 = fma((T)3, ch, ph);
+    const T v2 = fma((T)3, cl, nl), v3 = fma((T)3, ch, nh);
+    T* o = x + f;
     if (overwrite) {
-      o.x = v0;
-      o.y = v1;
+      o[0] = q * v0;
+      o[fy] = q * v1;
+      o[fz] = q * v2;
+      o[fz + fy] = q * v3;
     } else {
-      o = *px;
-      o.x += v0;
-      o.y += v1;
+      const T x0 = o[0], x1 = o[fy], x2 = o[fz], x3 = o[fz + fy];
+      o[0] = fma(q, v0, x0);
+      o[fy] = fma(q, v1, x1);
+      o[fz] = fma(q, v2, x2);
+      o[fz + fy] = fma(q, v3, x3);
     }
-    *px = o;
+    pl = cl;
+    ph = ch;
+    cl = nl;
+    ch = nh;
   }
 }
 
@@ -1058,18 +1177,28 @@ __global__ void __launch_bounds__(kChainThreads) k_coarse_chain(CoarseChain ch,
     reinterpret_cast<float4*>(x_out)[c] = reinterpret_cast<const float4*>(S.x)[c];
 }
 
-// x = P b on the coarsest level: one block, dense pseudo-inverse.
+// x = P b on the coarsest level, dense pseudo-inverse: one warp per row, the
+// lanes' partial sums combined by shuffles in a fixed order.
 template <typename T>
-__global__ void k_coarse_solve(const T* __restrict__ P, const T* __restrict__ b,
-                               T* __restrict__ x, int mc) {
-  __shared__ T sb[kMaxCoarse];
-  for (int q = threadIdx.x; q < mc; q += blockDim.x) sb[q] = b[q];
-  __syncthreads();
-  for (int r = threadIdx.x; r < mc; r += blockDim.x) {
-    T acc = 0;
-    for (int q = 0; q < mc; ++q) acc = fma(__ldg(P + (int64_t)r * mc + q), sb[q], acc);
-    x[r] = acc;
-  }
+__global__ void __launch_bounds__(256) k_coarse_solve(const T* __restrict__ P,
+                                                      const T* __restrict__ b, T* __restrict__ x,
+                                                      int mc) {
+  pdl_wait();
+  pdl_trigger();
+  const int lane = threadIdx.x & 31;
+  const int r = (blockIdx.x * 256 + threadIdx.x) >> 5;
+  if (r >= mc) return;
+  T acc = 0;
+  for (int q = lane; q < mc; q += 32) acc = fma(__ldg(P + (int64_t)r * mc + q), __ldg(b + q), acc);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) x[r] = acc;
+}
+
+template <typename T>
+void launch_coarse_solve(const T* P, const T* b, T* x, int mc, cudaStream_t s) {
+  count_launch();
+  launch_pdl(k_coarse_solve<T>, dim3(div_up(mc, 8)), dim3(256), 0, s, P, b, x, mc);
 }
 
 // Gauss-Jordan inverse with partial pivoting (host, n <= kMaxCoarse).
@@ -1137,7 +1266,7 @@ void pre_smooth(ibm_ctx* c, int l, const TB* b, T* bcopy, T* x, T* t, int p, cud
   const double h2 = L.h * L.h;
   const int two = p >= 2;
   const bool vec = std::is_same<T, float>::value && vec_ok(L.d);
-  const int zc = vec_zc(L.d);
+  const int zc = vec_zc(L.d), zm = zm_planes(L.d);
   const int ph = l == 0 ? prof_begin(c, IBM_PROF_MG_SMOOTH_FINE) : -1;
   count_launch();
   if constexpr (std::is_same<T, float>::value) {
@@ -1148,8 +1277,8 @@ void pre_smooth(ibm_ctx* c, int l, const TB* b, T* bcopy, T* x, T* t, int p, cud
   }
   if constexpr (!std::is_same<TB, float2>::value) {
     if (!vec)
-      k_first<T, TB><<<zm_grid(L.d), dim3(BX, BY), 0, s>>>(
-          L.d, b, bcopy, x, w_over_n<T>(w[0] * h2), w_over_n<T>(two ? w[1] : 0.0), (T)h2, two);
+      launch_pdl(k_first<T, TB>, zm_grid(L.d, zm), dim3(BX, BY), 0, s, L.d, b, bcopy, x,
+                 first_weights<T>(w[0], two ? w[1] : 0.0, h2), two, zm);
   }
   prof_end_or_note(c, ph, (double)L.m * (sizeof(TB) + sizeof(T) + (bcopy ? sizeof(T) : 0)));
   const T* bb = bcopy ? bcopy : reinterpret_cast<const T*>(b);
@@ -1166,8 +1295,8 @@ void pre_smooth(ibm_ctx* c, int l, const TB* b, T* bcopy, T* x, T* t, int p, cud
                    (const float*)cur, (const float*)bb, nxt, (float)w[q], (float)h2, zc);
     }
     if (!vec)
-      k_sweep<T, T, T><<<zm_grid(L.d), dim3(BX, BY), 0, s>>>(L.d, cur, bb, nxt,
-                                                            w_over_n<T>(w[q]), (T)h2);
+      launch_pdl(k_sweep<T, T, T>, zm_grid(L.d, zm), dim3(BX, BY), 0, s, L.d, (const T*)cur, bb,
+                 nxt, over_count<T>(w[q]), (T)h2, zm);
     T* tmp = cur; cur = nxt; nxt = tmp;
   }
   if (cur != x) {
@@ -1191,8 +1320,9 @@ void sweep_step(ibm_ctx* c, int l, const T* src, const T* b, TO* dst, double w, 
       return;
     }
   }
-  k_sweep<T, T, TO><<<zm_grid(L.d), dim3(BX, BY), 0, s>>>(L.d, src, b, dst, w_over_n<T>(w),
-                                                         (T)h2);
+  const int zm = zm_planes(L.d);
+  launch_pdl(k_sweep<T, T, TO>, zm_grid(L.d, zm), dim3(BX, BY), 0, s, L.d, src, b, dst,
+             over_count<T>(w), (T)h2, zm);
 }
 
 // Post-smoothing: p Chebyshev steps from x; the last step writes out (which
@@ -1254,9 +1384,12 @@ void coarse_correct(ibm_ctx* c, int l, const T* b, T* x, int pre, int post, cuda
       done = true;
     }
   }
+  // the one-cell transfers: a thread covers two fine rows and planes per step
+  const int zt = std::max(1, zm_planes(L.d) / 2);
+  const dim3 gt(div_up(L.d.nx, BX), div_up(C.d.ny, BY), div_up(C.d.nz, zt));
   if (!done)
-    k_restrict<T><<<dim3(div_up(C.d.nx, BX), div_up(C.d.ny, BY), div_up(C.d.nz, ZC / 2)),
-                    dim3(BX, BY), 0, s>>>(L.d, C.d, xin, b, cp.b, (T)(1.0 / (L.h * L.h)));
+    launch_pdl(k_restrict<T>, gt, dim3(BX, BY), 0, s, L.d, C.d, xin, b, cp.b,
+               (T)(1.0 / (L.h * L.h)), zt);
   prof_note(c, (double)L.m * ((xin ? 2 : 1) * sizeof(T)) + (double)C.m * sizeof(T));
   vcycle<T>(c, l + 1, cp.b, cp.x, cp.t, pre, post, s);
   done = false;
@@ -1270,8 +1403,8 @@ void coarse_correct(ibm_ctx* c, int l, const T* b, T* x, int pre, int post, cuda
     }
   }
   if (!done)
-    k_prolong<T><<<dim3(div_up(C.d.nx, BX), div_up(L.d.ny, BY), div_up(L.d.nz, ZC)),
-                   dim3(BX, BY), 0, s>>>(L.d, C.d, cp.x, x, pre > 0 ? 0 : 1);
+    launch_pdl(k_prolong<T>, gt, dim3(BX, BY), 0, s, L.d, C.d, (const T*)cp.x, x,
+               pre > 0 ? 0 : 1, zt);
   prof_note(c, (double)C.m * sizeof(T) + (double)L.m * ((pre > 0 ? 2 : 1) * sizeof(T)));
 }
 
@@ -1369,8 +1502,7 @@ void vcycle(ibm_ctx* c, int l, const T* b, T* x, T* t, int pre, int post, cudaSt
     if (l > 0 && chain_vcycle(c, l, b, x, pre, post, s)) return;
   }
   if (l == c->n_levels - 1) {
-    count_launch();
-    k_coarse_solve<T><<<1, 256, 0, s>>>(pinv_of<T>(c), b, x, c->coarse_m);
+    launch_coarse_solve<T>(pinv_of<T>(c), b, x, c->coarse_m, s);
     prof_note(c, (double)c->coarse_m * (c->coarse_m + 2) * sizeof(T));
     return;
   }
@@ -1458,8 +1590,7 @@ ibm_status mg_vcycle(ibm_ctx* c, const double* r, double* z, int prec, int pre, 
   MGLevel& L0 = c->lv[0];
   if (c->n_levels == 1) {
     // the whole grid is the coarsest level: the cycle is the exact pseudo-inverse
-    count_launch();
-    k_coarse_solve<double><<<1, 256, 0, s>>>(c->coarse_pinv64, r, z, c->coarse_m);
+    launch_coarse_solve<double>(c->coarse_pinv64, r, z, c->coarse_m, s);
     IBM_LAUNCH_CHECK(c);
     return IBM_OK;
   }
@@ -1481,8 +1612,9 @@ ibm_status mg_vcycle(ibm_ctx* c, const double* r, double* z, int prec, int pre, 
     } else {
       // only the rounded copy of r is needed (the zero iterate is never read)
       count_launch();
-      k_first<float, double><<<zm_grid(L0.d), dim3(BX, BY), 0, s>>>(
-          L0.d, r, L0.b32, L0.t32, w_over_n<float>(0.0), w_over_n<float>(0.0), 0.f, 0);
+      const int zm = zm_planes(L0.d);
+      k_first<float, double><<<zm_grid(L0.d, zm), dim3(BX, BY), 0, s>>>(L0.d, r, L0.b32, L0.t32,
+                                                                        FirstWeights<float>{}, 0, zm);
     }
     coarse_correct<float>(c, 0, L0.b32, L0.x32, pre, post, s);
     post_smooth<float, double>(c, 0, L0.b32, L0.x32, L0.t32, post, z, s);
