@@ -222,7 +222,8 @@ static void free_all(ibm_ctx* c) {
   cudaFree(m.t); cudaFree(m.t2); cudaFree(m.t32); cudaFree(m.dwf); cudaFree(m.dwc);
   cudaFree(m.wc32); cudaFree(m.cw32);
   cudaFree(m.cg);
-  cudaFree(m.t3); cudaFree(c->cg_scal);
+  cudaFree(m.t3); cudaFree(c->cg_bar);
+  cudaFree(m.c_val);
   cudaFree(m.entry_key); cudaFree(m.shell_cell); cudaFree(m.shell_off); cudaFree(m.ell_cell);
   cudaFree(m.ell_base); cudaFree(m.ell_len); cudaFree(m.ell_key); cudaFree(m.ell_coef);
   cudaFree(m.ell_coef32); cudaFree(m.ell_sw); cudaFree(m.ell_any);

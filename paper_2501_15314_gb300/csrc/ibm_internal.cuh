@@ -71,6 +71,14 @@ struct MarkerData {
   float* cw32 = nullptr;    // cw rounded to FP32
   double* cg = nullptr;     // [3][3n] conjugate-gradient work vectors for C^{-1}
   double* t3 = nullptr;     // [3][n] per-marker scratch (RHS_F in the C modes)
+  // rows of C = R^T R (cmode.cu), formed by the first C solve after the markers
+  // change: columns and the three components' values of marker k's row at
+  // c_off[k] .. c_off[k + 1]; c_n entries (0: the rows are not used)
+  bool c_formed = false;
+  int64_t c_n = 0, c_val_cap = 0;
+  int32_t* c_off = nullptr;     // [n + 1], after org
+  int32_t* c_col = nullptr;     // [c_n], after c_val
+  double* c_val = nullptr;      // [3][c_n]
   // cell-sorted (marker, slot) list for the atomic-free gathers
   int64_t n_entries = 0, entries_cap = 0;
   int32_t* entry_key = nullptr;   // marker * 64 + slot, sorted within a cell
@@ -185,7 +193,7 @@ struct ibm_ctx {
   double c_rtol = 1e-14;
   int c_maxit = 500;
   int64_t c_iters = 0;             // inner CG iterations since the call began
-  double* cg_scal = nullptr;       // [8] device scalars of the CG on C
+  unsigned* cg_bar = nullptr;      // [2] grid barrier of the CG on C
 
   // event timing of kernel classes (ibm_profile_enable)
   bool prof_on = false;
@@ -304,13 +312,10 @@ void launch_interp_dpos(ibm_ctx* c, const double* f, const double* m, double sca
                         bool accumulate, double* Xbar);
 // u[face] = beta * u[face] + scale * (R F)[face] on shell faces only
 void launch_shell_spread_faces(ibm_ctx* c, const double* F, double scale, double* u);
-// u = R F on the shell faces only (written, not accumulated)
-void launch_shell_spread_faces_set(ibm_ctx* c, const double* F, double* u);
 // Per-block partial L1 norms of R A and R B (2 doubles per block into part);
 // returns the number of blocks (0 without markers).
 int launch_shell_spread_asum2(ibm_ctx* c, const double* A, const double* B, double* part);
 // ---- C = R^T R (cmode.cu) ----
-void apply_C(ibm_ctx* c, const double* v, double* out);
 ibm_status c_solve(ibm_ctx* c, const double* t, double* s, double rtol, int maxit, int* iters);
 // the ctx's C mode from the options (and the CG counter reset)
 void set_cmode(ibm_ctx* c, const ibm_solve_opts* o);

@@ -445,7 +445,7 @@ __global__ void k_ell_fill(MkView mk, int64_t n_shell, const int32_t* __restrict
   if (live && lane % kEllLanes == 0) eany[q] = (uint8_t)any;
 }
 
-// u at the shell cells' lower faces += scale * (R F) (set: = scale * (R F)),
+// u at the shell cells' lower faces += scale * (R F),
 // faces outside every support left as they are: the spread through the
 // interleaved layout, kEllLanes lanes per cell (each its share of the
 // entries, summed by shuffles in a fixed order), the three components at
@@ -456,7 +456,7 @@ __global__ void k_shell_spread_ell(Dims d, int64_t n_shell, const int32_t* __res
                                    const int32_t* __restrict__ ekey,
                                    const double* __restrict__ esw,
                                    const uint8_t* __restrict__ eany, int64_t n_ell, int64_t nmk,
-                                   const double* __restrict__ F, double scale, int set,
+                                   const double* __restrict__ F, double scale,
                                    double* __restrict__ u) {
   const int64_t tq = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t g = tq >> 5;
@@ -517,7 +517,7 @@ __global__ void k_shell_spread_ell(Dims d, int64_t n_shell, const int32_t* __res
     const int64_t sy = d.nx + (dc == 0 ? 1 : 0);
     const int64_t sz = sy * (d.ny + (dc == 1 ? 1 : 0));
     const int64_t f = foff + ck * sz + cj * sy + ci;
-    u[f] = set ? scale * acc[dc] : fma(scale, acc[dc], u[f]);
+    u[f] = fma(scale, acc[dc], u[f]);
   }
 }
 
@@ -872,7 +872,7 @@ static ibm_status grow_markers(ibm_ctx* c, int64_t n) {
   m.cap = 0;
   const size_t ni = sizeof(int32_t) * 3 * n, nd = sizeof(double) * 9 * n;
   if (cudaMalloc(&m.bf, ni) != cudaSuccess || cudaMalloc(&m.bc, ni) != cudaSuccess ||
-      cudaMalloc(&m.org, ni) != cudaSuccess || cudaMalloc(&m.wf, nd) != cudaSuccess ||
+      cudaMalloc(&m.org, ni + sizeof(int32_t) * (n + 1)) != cudaSuccess || cudaMalloc(&m.wf, nd) != cudaSuccess ||
       cudaMalloc(&m.wc, nd) != cudaSuccess || cudaMalloc(&m.dwf, nd) != cudaSuccess ||
       cudaMalloc(&m.dwc, nd) != cudaSuccess ||
       cudaMalloc(&m.cw, sizeof(double) * 12 * n) != cudaSuccess ||
@@ -886,6 +886,7 @@ static ibm_status grow_markers(ibm_ctx* c, int64_t n) {
     cudaGetLastError();
     return set_err(c, IBM_ERR_NOMEM, "marker workspace allocation failed");
   }
+  m.c_off = m.org + 3 * n;
   m.cap = n;
   return IBM_OK;
 }
@@ -941,6 +942,7 @@ static ibm_status grow_ell(ibm_ctx* c, int64_t n_ell) {
 ibm_status markers_build(ibm_ctx* c, int64_t n, const double* X) {
   MarkerData& m = c->mk;
   c->markers_set = false;
+  m.c_formed = false;
   m.n = 0;
   m.n_entries = 0;
   m.n_shell = 0;
@@ -1144,7 +1146,7 @@ void launch_shell_spread_faces(ibm_ctx* c, const double* F, double scale, double
   count_launch();
   k_shell_spread_ell<<<div_up(32 * ell_groups(m.n_shell), TPB), TPB, 0, c->stream>>>(
       c->d, m.n_shell, m.ell_cell, m.ell_base, m.ell_len, m.ell_key, m.ell_sw, m.ell_any, m.n_ell,
-      m.n, F, scale, 0, u);
+      m.n, F, scale, u);
 }
 
 int launch_shell_spread_asum2(ibm_ctx* c, const double* A, const double* B, double* part) {
@@ -1154,15 +1156,6 @@ int launch_shell_spread_asum2(ibm_ctx* c, const double* A, const double* B, doub
   k_shell_spread_asum2<<<kSpreadAsumBlocks, TPB, 0, c->stream>>>(
       c->d, view(m), m.n_shell, m.shell_cell, m.shell_off, m.entry_key, A, B, part);
   return kSpreadAsumBlocks;
-}
-
-void launch_shell_spread_faces_set(ibm_ctx* c, const double* F, double* u) {
-  const MarkerData& m = c->mk;
-  if (m.n == 0 || m.n_shell == 0) return;
-  count_launch();
-  k_shell_spread_ell<<<div_up(32 * ell_groups(m.n_shell), TPB), TPB, 0, c->stream>>>(
-      c->d, m.n_shell, m.ell_cell, m.ell_base, m.ell_len, m.ell_key, m.ell_sw, m.ell_any, m.n_ell,
-      m.n, F, 1.0, 1, u);
 }
 
 }  // namespace ibm
