@@ -133,6 +133,22 @@ __device__ __forceinline__ dsf2 two_prod2(float2 a, float2 b) {
   const float2 p = __fmul2_rn(a, b);
   return {p, __ffma2_rn(a, b, neg2(p))};
 }
+// a + b, a * b for float2 b and a + b by Dekker's addition, per component
+__device__ __forceinline__ dsf2 ds_add_f2(dsf2 a, float2 b) {
+  dsf2 s = two_sum2(a.hi, b);
+  s.lo = __fadd2_rn(s.lo, a.lo);
+  return fast_two_sum2(s.hi, s.lo);
+}
+__device__ __forceinline__ dsf2 ds_mul_f2(dsf2 a, float2 b) {
+  dsf2 p = two_prod2(a.hi, b);
+  p.lo = __ffma2_rn(a.lo, b, p.lo);
+  return fast_two_sum2(p.hi, p.lo);
+}
+__device__ __forceinline__ dsf2 ds_add_d2(dsf2 a, dsf2 b) {
+  const dsf2 s = two_sum2(a.hi, b.hi);
+  return fast_two_sum2(s.hi, __fadd2_rn(s.lo, __fadd2_rn(a.lo, b.lo)));
+}
+__device__ __forceinline__ dsf2 ds_neg2(dsf2 a) { return {neg2(a.hi), neg2(a.lo)}; }
 // each component of a times the double-single b (dropping lo*lo), as ds_mul
 __device__ __forceinline__ dsf2 ds_mul2(dsf2 a, dsf b) {
   const float2 bh = make_float2(b.hi, b.hi), bl = make_float2(b.lo, b.lo);

@@ -152,12 +152,9 @@ struct ibm_ctx {
   double* f2 = nullptr;
   double* f3 = nullptr;
   double* f4 = nullptr;
-  float* g1 = nullptr;             // [nf] FP32 face temporaries (predictor)
-  float* g2 = nullptr;
-  float* g3 = nullptr;
-  float* g4 = nullptr;
-  float* g5 = nullptr;             // low parts of the predictor's residual
-  float* g6 = nullptr;             // the predictor's first correction, kept in FP32
+  float* hr = nullptr;             // predictor (faces by colour): the residual's
+  float* hl = nullptr;             // high and low parts,
+  float* he[2] = {nullptr, nullptr};   // two corrections
   double* red_part = nullptr;      // [kRedBlocks][kMaxRestart + 2] partials
   double* red_out = nullptr;       // [8][kMaxRestart + 2] reduced values
   // set by the step around its solve: the solver leaves the constant of the
@@ -248,7 +245,7 @@ ibm_status norm2_host(ibm_ctx* c, const double* x, int64_t n, double* out);
 ibm_status norm2_lead_host(ibm_ctx* c, const double* x, int64_t n, double* out);
 void launch_norm2_lead(const double* x, int64_t n, double* part, double* out, cudaStream_t s,
                        double* hout);
-// (a - nu Lap) u = rhs of Eq. (ustar) to o->helm_rtol; uses g1..g6
+// (a - nu Lap) u = rhs of Eq. (ustar) to o->helm_rtol; uses hr, hl, he
 ibm_status helmholtz_solve(ibm_ctx* c, const double* rhs, double* u, const ibm_solve_opts* o,
                            int* iters, double* relres);
 
@@ -271,20 +268,23 @@ void launch_grad_axpy(Dims d, const double* u_in, const double* p, double alpha,
 // out = alpha * G^T u + beta * c   (c may be null)
 void launch_gradt_axpby(Dims d, const double* u, double alpha, const double* c,
                         double beta, double* out, cudaStream_t s);
-// predictor helpers
-// (rhi, rlo) = (rhi, rlo) - A e in double-single (see k_helm_resid_ds) with
-// per-block sums of the new hi^2 in part[b * stride]; returns the block count
-int64_t launch_helm_resid_ds(Dims d, const float* e, float* rhi, float* rlo, double a,
-                             double nu_h2, double* part, int stride, cudaStream_t s);
-// number of floats of the predictor's padded FP32 face layout
+// predictor helpers (FP32 arrays by colour, see HelmGeom in stencil.cu)
+// number of floats of one such array
 int64_t helm_fp32_size(Dims d);
-// one FP32 Chebyshev step of the predictor (see k_helm_cheb_v4)
-void launch_helm_cheb(Dims d, const float* e, const float* eo, float* r32, float* rlo,
-                      const double* r64, double rs, float a, float nu_h2, float alpha, float beta,
-                      float* en, double* u, double us, int mode, cudaStream_t s,
-                      int flags = 0, const float* pe = nullptr, double ps = 0.0);
-// u = ps pe on the interior faces (pe on the predictor's padded FP32 layout)
-void launch_helm_flush(Dims d, const float* pe, double ps, double* u, cudaStream_t s);   // 1: e_old is zero; 2: u is zero (mode 2 writes it)
+// (rhi, rlo) = scale r64 (scale a power of two), e = D^{-1} r on colour 0
+void launch_helm_start(Dims d, const double* r64, float scale, double a, double nu_h2, float* rhi,
+                       float* rlo, float* e, cudaStream_t s);
+// one half-step of the cyclic Chebyshev iteration: colour col of e updated
+// from the other one with weight omega (old_zero: it is zero and not read)
+void launch_helm_half(Dims d, int col, float* e, const float* r, double a, double nu_h2,
+                      double omega, bool old_zero, cudaStream_t s);
+// (rhi, rlo) -= A e in double-single, per-block sums of the new hi^2 in part
+// (returns their number), D^{-1} of the new residual on colour 0 into en
+int64_t launch_helm_resid(Dims d, const float* e, float* rhi, float* rlo, double a, double nu_h2,
+                          float* en, double* part, cudaStream_t s);
+// u = 2^k (e + pe) (pe may be null), 0 on the walls; add: u += 2^k e
+void launch_helm_flush(Dims d, const float* e, const float* pe, int k, bool add, double* u,
+                       cudaStream_t s);
 // predictor RHS with the convective term of u_n fused in (with_adv != 0),
 // evaluated in double-single arithmetic (see k_predictor_rhs_ds)
 void launch_predictor_rhs_adv(Dims d, const double* u_n, const double* u_nm1,

@@ -528,291 +528,355 @@ __global__ void __launch_bounds__(BX * BY) k_predictor_rhs_ds(
   }
 }
 
-// FP32 work arrays of the predictor use a padded copy of the face layout:
-// rows padded to a multiple of 4 values, so that every row starts on a
-// 16-byte boundary and a thread can own four consecutive faces (one float4).
-// Padding holds 0 and is never read as a neighbour.
-struct FaceGeom32 {
-  int n[3][3];
-  int64_t off[3], sy[3], sz[3];
+// The predictor's FP32 work arrays hold the faces of a component by colour
+// (i + j + k even: colour 0, odd: colour 1), so that one colour of the
+// red-black Chebyshev steps below is contiguous: [component][colour][k][j][q],
+// q = i / 2, rows padded to a multiple of 4 values (16-byte alignment).  The
+// x-neighbours of element q of one colour are the elements q and q - 1 (i
+// even) or q and q + 1 (i odd) of the other colour's row, the y- and
+// z-neighbours its elements q of the rows beside.  Padding, and the wall face
+// i = nx of u_x when nx is odd, hold 0; when nx is even that face has no place.
+struct HelmGeom {
+  int nx;
+  int nq;              // elements per row and colour, ceil(nx / 2)
+  int n[3][3];         // faces per axis of each component
+  int64_t off[3], cs[3], sz[3];   // component, colour and plane strides
+  int64_t sy;          // row stride
 };
 
-FaceGeom32 make_face_geom32(Dims d) {
+HelmGeom make_helm_geom(Dims d) {
   const FaceGeom g = make_face_geom(d);
-  FaceGeom32 p;
+  HelmGeom p;
+  p.nx = d.nx;
+  p.nq = (d.nx + 1) / 2;
+  p.sy = (p.nq + 3) / 4 * 4;
   int64_t off = 0;
   for (int c = 0; c < 3; ++c) {
     for (int a = 0; a < 3; ++a) p.n[c][a] = g.n[c][a];
-    p.sy[c] = (g.n[c][0] + 3) / 4 * 4;
-    p.sz[c] = p.sy[c] * g.n[c][1];
+    p.sz[c] = p.sy * g.n[c][1];
+    p.cs[c] = p.sz[c] * g.n[c][2];
     p.off[c] = off;
-    off += p.sz[c] * g.n[c][2];
+    off += 2 * p.cs[c];
   }
   return p;
 }
 
-constexpr int HVY = 8;
 constexpr unsigned kFullMask = 0xffffffffu;
+constexpr int kHelmThreads = 256;
 
-// One FP32 Chebyshev step for A e = r on the padded layout, four faces per
-// thread; x-neighbours by shuffles, z by the march, y through L1.
-// mode 0: first step from e = 0: the normalised residual r^ = rs r is formed
-// in double-single from r64 (FP64, split without FP64 arithmetic) or, when
-// r64 is null, from the pair (r32, rlo) in place; r^ is kept in (r32, rlo)
-// and e_new = alpha r^.hi.  mode 1: e_new = e + beta (e - e_old) +
-// alpha (r - A e) with r = r32; mode 2: the same step, accumulated into the
-// FP64 iterate, u += us * e_new, and stored in e_new (the next residual
-// reads it).  The mode is a template parameter: each instance carries only
-// its own registers (mode 2 loads the FP64 iterate with the plane's other
-// inputs, so that its latency overlaps theirs).
-template <int mode>
-__global__ void __launch_bounds__(32 * HVY) k_helm_cheb_v4(
-    FaceGeom g, FaceGeom32 p, int zchunks, const float* __restrict__ e,
-    const float* __restrict__ eo, float* __restrict__ r32, float* __restrict__ rlo,
-    const double* __restrict__ r64, float rs_hi, float rs_lo, float a, float nu_h2, float alpha,
-    float beta, float* __restrict__ en, double* __restrict__ u, double us,
-    const float* __restrict__ pe, double ps, int flags) {
+// One of four weights by the number of ghost neighbours (0..3)
+__device__ __forceinline__ float by_ghosts(float4 w, int g) {
+  return g == 0 ? w.x : (g == 1 ? w.y : (g == 2 ? w.z : w.w));
+}
+
+// Ghost neighbours of a component's row or plane: a cell-centred axis has one
+// at each wall, the face-normal axis none.
+__device__ __forceinline__ int ghosts(bool centred, int x, int n) {
+  return centred ? (x == 0) + (x == n - 1) : 0;
+}
+
+// One half-step of the cyclic (red-black) Chebyshev iteration for A e = r:
+// the faces of colour col are updated in place from the other colour,
+//   e <- e + omega (D^{-1} (r + N e_other) - e),   A = D - N,
+// as e = w (r + nu s) + (1 - omega) e with s the neighbour sum and
+// w = omega / D (by ghost count).  The iterates of both colours at steps n and
+// n + 1 are those of the full Chebyshev iteration on D^{-1} A (half of its
+// values each), so a full iteration's convergence takes half its work
+// (Golub and Varga's cyclic Chebyshev semi-iterative method).
+// Four elements per thread (float4), LX threads per row, z-neighbours from the
+// march, x by one shuffle, y through L1.  old_zero: e of this colour is zero
+// and not read.  Weights are 0 at wall faces and past a row's end, where e is
+// and stays 0.  FULL: nx is a multiple of 8, so only the first and last element
+// of a row can differ from the row's others.  Bound by HBM and instruction
+// issue: 16 B per updated face, 8 B per face of the grid.
+template <int LX, bool FULL>
+__global__ void __launch_bounds__(kHelmThreads) k_helm_half(HelmGeom p, int zc, int zchunks,
+                                                            int col, float* e,
+                                                            const float* __restrict__ r, float nu,
+                                                            float4 w, float omw, int old_zero) {
   pdl_wait();
   pdl_trigger();
-  // flags: 1 = e_old is zero (not read); 2 = the FP64 iterate is not read
-  // (mode 2 writes u = us e_new + ps pe on every face, ps pe being a
-  // correction not yet added (none when pe is null), 0 on the wall faces)
-  const bool eo_zero = flags & 1, u_zero = flags & 2;
+  constexpr int kRows = kHelmThreads / LX;
   const int c = blockIdx.z / zchunks;
-  const int zc = blockIdx.z - c * zchunks;
-  const int lane = threadIdx.x;
-  const int x0 = 4 * (blockIdx.x * 32 + lane);
-  const int j = blockIdx.y * HVY + threadIdx.y;
-  const int n0 = sel3(c, p.n[0][0], p.n[1][0], p.n[2][0]);
+  const int z0 = (blockIdx.z - c * zchunks) * zc;
   const int n1 = sel3(c, p.n[0][1], p.n[1][1], p.n[2][1]);
   const int n2 = sel3(c, p.n[0][2], p.n[1][2], p.n[2][2]);
-  const int z0 = zc * ZH;
-  if (z0 >= n2 || blockIdx.x * 128 >= n0 || blockIdx.y * HVY >= n1) return;   // block-uniform
-  const int z1 = min(z0 + ZH, n2);
-  const bool act = x0 < n0 && j < n1;
-  const int64_t sy = sel3(c, p.sy[0], p.sy[1], p.sy[2]), sz = sel3(c, p.sz[0], p.sz[1], p.sz[2]);
-  int64_t f = sel3(c, p.off[0], p.off[1], p.off[2]) + (int64_t)z0 * sz + (int64_t)j * sy + x0;
-  const int64_t sy64 = sel3(c, g.sy[0], g.sy[1], g.sy[2]);
-  const int64_t sz64 = sel3(c, g.sz[0], g.sz[1], g.sz[2]);
-  int64_t f64 = sel3(c, g.off[0], g.off[1], g.off[2]) + (int64_t)z0 * sz64 + (int64_t)j * sy64 + x0;
+  if (z0 >= n2 || (int)blockIdx.y * kRows >= n1) return;   // block-uniform
+  const int z1 = min(z0 + zc, n2);
+  const int tx = threadIdx.x;
+  const int j = blockIdx.y * kRows + threadIdx.y;
+  const int q0 = 4 * (blockIdx.x * LX + tx);
+  const bool act = q0 < p.nq && j < n1;
+  const int64_t cs = sel3(c, p.cs[0], p.cs[1], p.cs[2]), sz = sel3(c, p.sz[0], p.sz[1], p.sz[2]);
+  const int64_t base = sel3(c, p.off[0], p.off[1], p.off[2]) + (int64_t)z0 * sz +
+                       (int64_t)j * p.sy + q0;
+  const float* eo = e + base + (1 - col) * cs;
+  float* ec = e + base + col * cs;
+  const float* rc = r + base + col * cs;
   const float4 Z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  // per-element validity and x-wall status
-  bool val[4], wallx[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    val[q] = act && (x0 + q < n0);
-    wallx[q] = c == 0 && (x0 + q == 0 || x0 + q == n0 - 1);
-  }
+  auto ld = [](const float* q) { return *reinterpret_cast<const float4*>(q); };
+  const bool hym = act && j > 0, hyp = act && j < n1 - 1;
+  const bool old_in = act && !old_zero;
+  // weights off and on the z-walls, of ordinary faces and of those with an
+  // x-ghost
+  const int gy = ghosts(c != 1, j, n1);
   const bool wally = c == 1 && (j == 0 || j == n1 - 1);
-  if constexpr (mode == 0) {
-    const dsf rs = {rs_hi, rs_lo};
-    for (int z = z0; z < z1; ++z, f += sz, f64 += sz64) {
-      const bool wallz = c == 2 && (z == 0 || z == n2 - 1);
-      float h4[4] = {0.f, 0.f, 0.f, 0.f}, l4[4] = {0.f, 0.f, 0.f, 0.f};
-      if (act && !r64) {
-        const float4 a4 = *reinterpret_cast<const float4*>(r32 + f);
-        const float4 b4 = *reinterpret_cast<const float4*>(rlo + f);
-        h4[0] = a4.x; h4[1] = a4.y; h4[2] = a4.z; h4[3] = a4.w;
-        l4[0] = b4.x; l4[1] = b4.y; l4[2] = b4.z; l4[3] = b4.w;
-      }
-      float rh[4], rl[4];
+  const float w_in = wally ? 0.f : by_ghosts(w, gy), w_in_x = wally ? 0.f : by_ghosts(w, gy + 1);
+  const float w_z = (wally || c == 2) ? 0.f : by_ghosts(w, gy + 1);
+  const float w_z_x = (wally || c == 2) ? 0.f : by_ghosts(w, gy + 2);
+  // per parity s of i the elements with an x-ghost and the dead ones
+  int ghost = 0, dead = 0;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const bool live = val[q] && !wallx[q] && !wally && !wallz;
-        dsf v = {0.f, 0.f};
-        if (live) v = ds_mul(r64 ? split_exact(__ldg(r64 + f64 + q)) : dsf{h4[q], l4[q]}, rs);
-        rh[q] = v.hi;
-        rl[q] = v.lo;
-      }
-      if (act) {
-        *reinterpret_cast<float4*>(r32 + f) = make_float4(rh[0], rh[1], rh[2], rh[3]);
-        *reinterpret_cast<float4*>(rlo + f) = make_float4(rl[0], rl[1], rl[2], rl[3]);
-        *reinterpret_cast<float4*>(en + f) =
-            make_float4(alpha * rh[0], alpha * rh[1], alpha * rh[2], alpha * rh[3]);
-      }
-    }
-    return;
+  for (int b = 0; b < 8; ++b) {
+    const int i = 2 * (q0 + (b & 3)) + (b >> 2);
+    if (c != 0 && (i == 0 || i == p.nx - 1)) ghost |= 1 << b;
+    if (i >= p.nx || (c == 0 && i == 0)) dead |= 1 << b;
   }
-  // ghost counts along y and z (cell-centred axes only), x per element
-  const int gy = (c != 1) ? ((j == 0) + (j == n1 - 1)) : 0;
-  int gx[4];
+  int s = (col + j + z0) & 1;   // i = 2 q + s
+  float4 om = (act && z0 > 0) ? ld(eo - sz) : Z4;
+  float4 oc = act ? ld(eo) : Z4;
+  for (int z = z0; z < z1; ++z) {
+    const float4 on = (act && z + 1 < n2) ? ld(eo + sz) : Z4;
+    const float4 ym = hym ? ld(eo - p.sy) : Z4;
+    const float4 yp = hyp ? ld(eo + p.sy) : Z4;
+    const float4 rr = act ? ld(rc) : Z4;
+    const float4 old = old_in ? ld(ec) : Z4;
+    // the x-neighbour outside the group: below (s = 0) or above (s = 1)
+    float side = __shfl_sync(kFullMask, s ? oc.x : oc.w, s ? tx + 1 : tx - 1, LX);
+    if (tx == (s ? LX - 1 : 0))
+      side = (act && (s ? q0 + 4 < p.nq : q0 > 0)) ? eo[s ? 4 : -1] : 0.f;
+    const bool zw = z == 0 || z == n2 - 1;
+    const float w0 = zw ? w_z : w_in, wx = zw ? w_z_x : w_in_x;
+    const int sp = s ? 4 : 0;
+    float wt[4] = {w0, w0, w0, w0};
+    auto special = [&](int t) {
+      if ((ghost >> (sp + t)) & 1) wt[t] = wx;
+      if ((dead >> (sp + t)) & 1) wt[t] = 0.f;
+    };
+    if (FULL) {
+      special(0);
+      special(3);
+    } else {
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
-    gx[q] = (c != 0) ? ((x0 + q == 0) + (x0 + q == n0 - 1)) : 0;
-  const bool has_ym = j > 0, has_yp = j < n1 - 1;
-  float4 ep = (act && z0 > 0) ? *reinterpret_cast<const float4*>(e + f - sz) : Z4;
-  float4 ec = act ? *reinterpret_cast<const float4*>(e + f) : Z4;
-  for (int z = z0; z < z1; ++z, f += sz, f64 += sz64) {
-    const float4 ez = (act && z + 1 < n2) ? *reinterpret_cast<const float4*>(e + f + sz) : Z4;
-    const float4 ym = (act && has_ym) ? *reinterpret_cast<const float4*>(e + f - sy) : Z4;
-    const float4 yp = (act && has_yp) ? *reinterpret_cast<const float4*>(e + f + sy) : Z4;
-    const float4 rr = act ? *reinterpret_cast<const float4*>(r32 + f) : Z4;
-    const float4 eold = (act && !eo_zero) ? *reinterpret_cast<const float4*>(eo + f) : Z4;
-    float left = __shfl_up_sync(kFullMask, ec.w, 1);
-    float right = __shfl_down_sync(kFullMask, ec.x, 1);
-    if (lane == 0) left = (act && x0 > 0) ? e[f - 1] : 0.f;
-    if (lane == 31) right = (act && x0 + 4 < n0) ? e[f + 4] : 0.f;
-    const bool wallz = c == 2 && (z == 0 || z == n2 - 1);
-    const int gz = (c != 2) ? ((z == 0) + (z == n2 - 1)) : 0;
-    double uo[4] = {0.0, 0.0, 0.0, 0.0};
-    float4 pv = Z4;
-    if constexpr (mode == 2) {
-      if (u_zero) {
-        if (pe && act) pv = *reinterpret_cast<const float4*>(pe + f);
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (val[q] && !wallx[q] && !wally && !wallz) uo[q] = u[f64 + q];
-      }
+      for (int t = 0; t < 4; ++t) special(t);
     }
-    const float ev[4] = {ec.x, ec.y, ec.z, ec.w};
-    const float evp[4] = {ep.x, ep.y, ep.z, ep.w};
-    const float evn[4] = {ez.x, ez.y, ez.z, ez.w};
-    const float vym[4] = {ym.x, ym.y, ym.z, ym.w};
-    const float vyp[4] = {yp.x, yp.y, yp.z, yp.w};
-    const float vr[4] = {rr.x, rr.y, rr.z, rr.w};
-    const float vo[4] = {eold.x, eold.y, eold.z, eold.w};
-    float out[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int x = x0 + q;
-      float sx = 0.f;
-      // x-neighbours exist inside the row; on a cell-centred x-axis the
-      // missing ones are ghosts (counted in gx), on the face axis the wall
-      // faces hold 0
-      if (x > 0) sx += (q == 0) ? left : ev[q - 1];
-      if (x < n0 - 1) sx += (q == 3) ? right : ev[q + 1];
-      const float s = sx + (vym[q] + vyp[q]) + (evp[q] + evn[q]);
-      const float diag = a + nu_h2 * (float)(6 + gx[q] + gy + gz);
-      const float res = vr[q] - fmaf(diag, ev[q], -nu_h2 * s);
-      const bool live = val[q] && !wallx[q] && !wally && !wallz;
-      out[q] = live ? ev[q] + beta * (ev[q] - vo[q]) + alpha * res : 0.f;
-    }
-    if (act) *reinterpret_cast<float4*>(en + f) = make_float4(out[0], out[1], out[2], out[3]);
-    if constexpr (mode == 2) {
-      const float pq[4] = {pv.x, pv.y, pv.z, pv.w};
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        // (the same products and roundings as adding ps pe first, then us e_new)
-        if (u_zero && pe) uo[q] = ps * f2d_exact(pq[q]);
-        if (val[q] && !wallx[q] && !wally && !wallz)
-          u[f64 + q] = u_zero && !pe ? us * f2d_exact(out[q])
-                                     : fma(us, f2d_exact(out[q]), uo[q]);   // widened without the FP64 pipe
-        else if (u_zero && val[q])
-          u[f64 + q] = 0.0;
-      }
-    }
-    ep = ec;
-    ec = ez;
+    float4 o;
+    o.x = fmaf(wt[0], fmaf(nu, (oc.x + (s ? oc.y : side)) + (ym.x + yp.x) + (om.x + on.x), rr.x),
+               omw * old.x);
+    o.y = fmaf(wt[1], fmaf(nu, (oc.y + (s ? oc.z : oc.x)) + (ym.y + yp.y) + (om.y + on.y), rr.y),
+               omw * old.y);
+    o.z = fmaf(wt[2], fmaf(nu, (oc.z + (s ? oc.w : oc.y)) + (ym.z + yp.z) + (om.z + on.z), rr.z),
+               omw * old.z);
+    o.w = fmaf(wt[3], fmaf(nu, (oc.w + (s ? side : oc.z)) + (ym.w + yp.w) + (om.w + on.w), rr.w),
+               omw * old.w);
+    if (act) *reinterpret_cast<float4*>(ec) = o;
+    om = oc;
+    oc = on;
+    eo += sz;
+    ec += sz;
+    rc += sz;
+    s ^= 1;
   }
 }
 
-// Next normalised residual of the predictor's defect correction, in
-// double-single arithmetic on the FP32 pipes: after a correction that solved
-// A e = r^ (r^ = r / ||r|| held as the pair (rhi, rlo)) and added ||r|| e to
-// the FP64 iterate, the new residual is ||r|| (r^ - A e).  This kernel forms
-// q = r^ - A e exactly enough (A e of the FP32 e with error-free sums and
-// products, the last two sums by Dekker's addition: a few units of 2^-46
-// relative to r^) and writes it back to (rhi, rlo); the
-// block's sum of q.hi^2 goes to part[block * stride] (every block writes
-// one).  The FP64 pipe is not used.
-__global__ void __launch_bounds__(32 * HVY) k_helm_resid_ds(
-    FaceGeom32 p, int zchunks, const float* __restrict__ e, float* __restrict__ rhi,
-    float* __restrict__ rlo, float a_hi, float a_lo, float nu_hi, float nu_lo,
-    double* __restrict__ part, int stride) {
+// Start of the solve: the residual r^ = scale r (scale a power of two: exact)
+// of the FP64 right-hand side as FP32 pairs (split_exact) by colour, and the
+// first half-step e_0 = D^{-1} r^ of colour 0.  One face per thread, so that a
+// warp reads 32 consecutive FP64 values and writes two whole 64-byte pieces.
+__global__ void __launch_bounds__(kHelmThreads) k_helm_start(FaceGeom g, HelmGeom p, int zc,
+                                                             int zchunks,
+                                                             const double* __restrict__ r64,
+                                                             float scale, float4 dinv,
+                                                             float* __restrict__ rhi,
+                                                             float* __restrict__ rlo,
+                                                             float* __restrict__ e) {
   const int c = blockIdx.z / zchunks;
-  const int zc = blockIdx.z - c * zchunks;
-  const int lane = threadIdx.x;
-  const int x0 = 4 * (blockIdx.x * 32 + lane);
-  const int j = blockIdx.y * HVY + threadIdx.y;
-  const int n0 = sel3(c, p.n[0][0], p.n[1][0], p.n[2][0]);
+  const int z0 = (blockIdx.z - c * zchunks) * zc;
   const int n1 = sel3(c, p.n[0][1], p.n[1][1], p.n[2][1]);
   const int n2 = sel3(c, p.n[0][2], p.n[1][2], p.n[2][2]);
-  const int z0 = zc * ZH;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= 2 * p.nq || j >= n1) return;
+  const int z1 = min(z0 + zc, n2);
+  const int64_t cs = sel3(c, p.cs[0], p.cs[1], p.cs[2]), sz = sel3(c, p.sz[0], p.sz[1], p.sz[2]);
+  const int64_t sz64 = sel3(c, g.sz[0], g.sz[1], g.sz[2]);
+  const double* src = r64 + sel3(c, g.off[0], g.off[1], g.off[2]) +
+                      (int64_t)j * sel3(c, g.sy[0], g.sy[1], g.sy[2]) + i;
+  const int64_t base = sel3(c, p.off[0], p.off[1], p.off[2]) + (int64_t)j * p.sy + (i >> 1);
+  const bool live = i < p.nx && !(c == 0 && i == 0) && !(c == 1 && (j == 0 || j == n1 - 1));
+  const int gxy = ghosts(c != 0, i, p.nx) + ghosts(c != 1, j, n1);
+#pragma unroll 4
+  for (int z = z0; z < z1; ++z) {
+    dsf v = {0.f, 0.f};
+    if (live && !(c == 2 && (z == 0 || z == n2 - 1)))
+      v = split_exact(__ldg(src + (int64_t)z * sz64));
+    v.hi *= scale;
+    v.lo *= scale;
+    const int col = (i + j + z) & 1;
+    const int64_t f = base + (int64_t)z * sz + col * cs;
+    rhi[f] = v.hi;
+    rlo[f] = v.lo;
+    if (col == 0) e[f] = by_ghosts(dinv, gxy + ghosts(c != 2, z, n2)) * v.hi;
+  }
+}
+
+// (rhi, rlo) <- (rhi, rlo) - A e in double-single arithmetic on the FP32
+// pipes: after the FP32 correction e the new residual q = r^ - A e, formed
+// exactly enough (A e with error-free sums and products, the last two sums by
+// Dekker's addition: a few units of 2^-46 relative to r^); the block's sum of
+// q.hi^2 goes to part[block] (every block writes one).  The first half-step of
+// the next correction, D^{-1} q on colour 0, goes to en.  Two elements of each
+// colour per thread.  The FP64 pipe is not used.
+template <int LX>
+__global__ void __launch_bounds__(kHelmThreads) k_helm_resid(
+    HelmGeom p, int zc, int zchunks, const float* __restrict__ e, float* __restrict__ rhi,
+    float* __restrict__ rlo, dsf A, dsf NU, float4 dinv, float* __restrict__ en,
+    double* __restrict__ part) {
+  constexpr int kRows = kHelmThreads / LX;
+  const int c = blockIdx.z / zchunks;
+  const int z0 = (blockIdx.z - c * zchunks) * zc;
+  const int n1 = sel3(c, p.n[0][1], p.n[1][1], p.n[2][1]);
+  const int n2 = sel3(c, p.n[0][2], p.n[1][2], p.n[2][2]);
   const int64_t blk = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  if (z0 >= n2 || blockIdx.x * 128 >= n0 || blockIdx.y * HVY >= n1) {   // block-uniform
-    if (threadIdx.x == 0 && threadIdx.y == 0) part[blk * stride] = 0.0;
+  if (z0 >= n2 || (int)blockIdx.y * kRows >= n1) {   // block-uniform
+    if (threadIdx.x == 0 && threadIdx.y == 0) part[blk] = 0.0;
     return;
   }
-  const int z1 = min(z0 + ZH, n2);
-  const bool act = x0 < n0 && j < n1;
-  const int64_t sy = sel3(c, p.sy[0], p.sy[1], p.sy[2]), sz = sel3(c, p.sz[0], p.sz[1], p.sz[2]);
-  int64_t f = sel3(c, p.off[0], p.off[1], p.off[2]) + (int64_t)z0 * sz + (int64_t)j * sy + x0;
-  const float4 Z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  bool val[4], wallx[4];
-  int gx[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    val[q] = act && (x0 + q < n0);
-    wallx[q] = c == 0 && (x0 + q == 0 || x0 + q == n0 - 1);
-    gx[q] = (c != 0) ? ((x0 + q == 0) + (x0 + q == n0 - 1)) : 0;
-  }
+  const int z1 = min(z0 + zc, n2);
+  const int tx = threadIdx.x;
+  const int j = blockIdx.y * kRows + threadIdx.y;
+  const int q0 = 2 * (blockIdx.x * LX + tx);
+  const bool act = q0 < p.nq && j < n1;
+  const int64_t cs = sel3(c, p.cs[0], p.cs[1], p.cs[2]), sz = sel3(c, p.sz[0], p.sz[1], p.sz[2]);
+  const int64_t base = sel3(c, p.off[0], p.off[1], p.off[2]) + (int64_t)j * p.sy + q0;
+  const bool hym = act && j > 0, hyp = act && j < n1 - 1;
+  const int gy = ghosts(c != 1, j, n1);
   const bool wally = c == 1 && (j == 0 || j == n1 - 1);
-  const int gy = (c != 1) ? ((j == 0) + (j == n1 - 1)) : 0;
-  const bool has_ym = j > 0, has_yp = j < n1 - 1;
-  const dsf A = {a_hi, a_lo}, NU = {nu_hi, nu_lo};
+  const float2 Z2 = make_float2(0.f, 0.f);
+  auto ld = [](const float* q) { return *reinterpret_cast<const float2*>(q); };
   const dsf D6 = ds_add(A, ds_mul_f(NU, 6.f));
   float acc = 0.f;
-  float4 ep = (act && z0 > 0) ? *reinterpret_cast<const float4*>(e + f - sz) : Z4;
-  float4 ec = act ? *reinterpret_cast<const float4*>(e + f) : Z4;
-  for (int z = z0; z < z1; ++z, f += sz) {
-    const float4 ez = (act && z + 1 < n2) ? *reinterpret_cast<const float4*>(e + f + sz) : Z4;
-    const float4 ym = (act && has_ym) ? *reinterpret_cast<const float4*>(e + f - sy) : Z4;
-    const float4 yp = (act && has_yp) ? *reinterpret_cast<const float4*>(e + f + sy) : Z4;
-    const float4 rh = act ? *reinterpret_cast<const float4*>(rhi + f) : Z4;
-    const float4 rl = act ? *reinterpret_cast<const float4*>(rlo + f) : Z4;
-    float left = __shfl_up_sync(kFullMask, ec.w, 1);
-    float right = __shfl_down_sync(kFullMask, ec.x, 1);
-    if (lane == 0) left = (act && x0 > 0) ? e[f - 1] : 0.f;
-    if (lane == 31) right = (act && x0 + 4 < n0) ? e[f + 4] : 0.f;
-    const bool wallz = c == 2 && (z == 0 || z == n2 - 1);
-    const int gz = (c != 2) ? ((z == 0) + (z == n2 - 1)) : 0;
-    const float ev[4] = {ec.x, ec.y, ec.z, ec.w};
-    const float evp[4] = {ep.x, ep.y, ep.z, ep.w};
-    const float evn[4] = {ez.x, ez.y, ez.z, ez.w};
-    const float vym[4] = {ym.x, ym.y, ym.z, ym.w};
-    const float vyp[4] = {yp.x, yp.y, yp.z, yp.w};
-    const float vrh[4] = {rh.x, rh.y, rh.z, rh.w};
-    const float vrl[4] = {rl.x, rl.y, rl.z, rl.w};
-    float oh[4], ol[4];
+  int64_t f = base + (int64_t)z0 * sz;
+  // both colours at the planes below, at and above
+  float2 em[2], ec[2], ez[2];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int x = x0 + q;
-      const float xl = (x > 0) ? ((q == 0) ? left : ev[q - 1]) : 0.f;
-      const float xr = (x < n0 - 1) ? ((q == 3) ? right : ev[q + 1]) : 0.f;
-      dsf s = two_sum(xl, xr);
-      s = ds_add_f(s, vym[q]);
-      s = ds_add_f(s, vyp[q]);
-      s = ds_add_f(s, evp[q]);
-      s = ds_add_f(s, evn[q]);
-      const int gh = gx[q] + gy + gz;
-      const dsf diag = gh == 0 ? D6 : ds_add(A, ds_mul_f(NU, (float)(6 + gh)));
-      const dsf Ae = ds_add_d(ds_mul_f(diag, ev[q]), ds_neg(ds_mul(NU, s)));
-      dsf qv = ds_add_d(dsf{vrh[q], vrl[q]}, ds_neg(Ae));
-      const bool live = val[q] && !wallx[q] && !wally && !wallz;
-      if (!live) qv = dsf{0.f, 0.f};
-      oh[q] = qv.hi;
-      ol[q] = qv.lo;
-      acc = fmaf(qv.hi, qv.hi, acc);
+  for (int k = 0; k < 2; ++k) {
+    em[k] = (act && z0 > 0) ? ld(e + f + k * cs - sz) : Z2;
+    ec[k] = act ? ld(e + f + k * cs) : Z2;
+  }
+  for (int z = z0; z < z1; ++z, f += sz) {
+    float2 ym[2], yp[2], rh[2], rl[2];
+    float side[2];   // x-neighbour of the colour's own group among the other's
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int64_t fk = f + k * cs;
+      ez[k] = (act && z + 1 < n2) ? ld(e + fk + sz) : Z2;
+      ym[k] = hym ? ld(e + fk - p.sy) : Z2;
+      yp[k] = hyp ? ld(e + fk + p.sy) : Z2;
+      rh[k] = act ? ld(rhi + fk) : Z2;
+      rl[k] = act ? ld(rlo + fk) : Z2;
+      const int o = 1 - k, s = (k + j + z) & 1;
+      side[k] = __shfl_sync(kFullMask, s ? ec[o].x : ec[o].y, s ? tx + 1 : tx - 1, LX);
+      if (tx == (s ? LX - 1 : 0))
+        side[k] = (act && (s ? q0 + 2 < p.nq : q0 > 0)) ? e[f + o * cs + (s ? 2 : -1)] : 0.f;
     }
-    if (act) {
-      *reinterpret_cast<float4*>(rhi + f) = make_float4(oh[0], oh[1], oh[2], oh[3]);
-      *reinterpret_cast<float4*>(rlo + f) = make_float4(ol[0], ol[1], ol[2], ol[3]);
+    const bool wall = wally || (c == 2 && (z == 0 || z == n2 - 1));
+    const int gyz = gy + ghosts(c != 2, z, n2);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int o = 1 - k, s = (k + j + z) & 1;
+      const float2 xb = make_float2(s ? ec[o].y : side[k], s ? side[k] : ec[o].x);
+      dsf2 sm = two_sum2(ec[o], xb);
+      sm = ds_add_f2(sm, ym[o]);
+      sm = ds_add_f2(sm, yp[o]);
+      sm = ds_add_f2(sm, em[o]);
+      sm = ds_add_f2(sm, ez[o]);
+      const int i0 = 2 * q0 + s, i1 = i0 + 2;
+      const int g0 = gyz + ghosts(c != 0, i0, p.nx), g1 = gyz + ghosts(c != 0, i1, p.nx);
+      dsf d0 = D6, d1 = D6;
+      if (g0 > 0) d0 = ds_add(A, ds_mul_f(NU, (float)(6 + g0)));
+      if (g1 > 0) d1 = ds_add(A, ds_mul_f(NU, (float)(6 + g1)));
+      const dsf2 diag = {make_float2(d0.hi, d1.hi), make_float2(d0.lo, d1.lo)};
+      const dsf2 Ae = ds_add_d2(ds_mul_f2(diag, ec[k]), ds_neg2(ds_mul2(sm, NU)));
+      dsf2 v = ds_add_d2(dsf2{rh[k], rl[k]}, ds_neg2(Ae));
+      if (wall || i0 >= p.nx || (c == 0 && i0 == 0)) v.hi.x = v.lo.x = 0.f;
+      if (wall || i1 >= p.nx) v.hi.y = v.lo.y = 0.f;
+      acc = fmaf(v.hi.x, v.hi.x, acc);
+      acc = fmaf(v.hi.y, v.hi.y, acc);
+      if (act) {
+        const int64_t fk = f + k * cs;
+        *reinterpret_cast<float2*>(rhi + fk) = v.hi;
+        *reinterpret_cast<float2*>(rlo + fk) = v.lo;
+        if (k == 0)
+          *reinterpret_cast<float2*>(en + fk) =
+              make_float2(by_ghosts(dinv, g0) * v.hi.x, by_ghosts(dinv, g1) * v.hi.y);
+      }
     }
-    ep = ec;
-    ec = ez;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      em[k] = ec[k];
+      ec[k] = ez[k];
+    }
   }
   // block reduction (FP64, fixed order)
   double v = (double)acc;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFullMask, v, o);
-  __shared__ double sh[HVY];
-  if (lane == 0) sh[threadIdx.y] = v;
+  __shared__ double sh[kHelmThreads / 32];
+  const int tid = threadIdx.y * LX + tx;
+  if ((tid & 31) == 0) sh[tid >> 5] = v;
   __syncthreads();
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
+  if (tid == 0) {
     double t = 0.0;
-    for (int w = 0; w < HVY; ++w) t += sh[w];
-    part[blk * stride] = t;
+    for (int k = 0; k < kHelmThreads / 32; ++k) t += sh[k];
+    part[blk] = t;
+  }
+}
+
+// v 2^k by its exponent field (v 0 or normal, and so the result)
+__device__ __forceinline__ double scale_exp(double v, int k) {
+  return v == 0.0 ? v : __longlong_as_double(__double_as_longlong(v) + ((long long)k << 52));
+}
+
+// Corrections into the FP64 iterate on the faces' own layout: u = 2^k (pe + e)
+// (pe null: 2^k e), 0 on the wall faces; ADD: u += 2^k e on the interior
+// faces.  The FP32 values are widened with integer operations and the scale
+// moves exponents only, so a face costs the FP64 pipe one addition.
+// One face per thread (as k_helm_start).
+template <bool ADD>
+__global__ void __launch_bounds__(kHelmThreads) k_helm_flush(FaceGeom g, HelmGeom p, int zc,
+                                                             int zchunks,
+                                                             const float* __restrict__ e,
+                                                             const float* __restrict__ pe, int k,
+                                                             double* __restrict__ u) {
+  const int c = blockIdx.z / zchunks;
+  const int z0 = (blockIdx.z - c * zchunks) * zc;
+  const int n1 = sel3(c, p.n[0][1], p.n[1][1], p.n[2][1]);
+  const int n2 = sel3(c, p.n[0][2], p.n[1][2], p.n[2][2]);
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= p.nx || j >= n1) return;
+  const int z1 = min(z0 + zc, n2);
+  const int64_t cs = sel3(c, p.cs[0], p.cs[1], p.cs[2]), sz = sel3(c, p.sz[0], p.sz[1], p.sz[2]);
+  const int64_t sz64 = sel3(c, g.sz[0], g.sz[1], g.sz[2]);
+  double* dst = u + sel3(c, g.off[0], g.off[1], g.off[2]) +
+                (int64_t)j * sel3(c, g.sy[0], g.sy[1], g.sy[2]) + i;
+  const int64_t base = sel3(c, p.off[0], p.off[1], p.off[2]) + (int64_t)j * p.sy + (i >> 1);
+  const bool live = !(c == 0 && i == 0) && !(c == 1 && (j == 0 || j == n1 - 1));
+  const bool wall_next = c == 0 && i == p.nx - 1;   // u_x's wall face i = nx
+#pragma unroll 4
+  for (int z = z0; z < z1; ++z) {
+    const int64_t f = base + (int64_t)z * sz + ((i + j + z) & 1) * cs;
+    double* d = dst + (int64_t)z * sz64;
+    const bool in = live && !(c == 2 && (z == 0 || z == n2 - 1));
+    if (ADD) {
+      if (in) *d += scale_exp(f2d_exact(e[f]), k);
+    } else {
+      double v = f2d_exact(e[f]);
+      if (pe) v += f2d_exact(pe[f]);
+      *d = in ? scale_exp(v, k) : 0.0;
+      if (wall_next) d[1] = 0.0;
+    }
   }
 }
 
@@ -896,96 +960,85 @@ void launch_gradient_t(Dims d, const double* u, double* out, double inv_h, cudaS
   launch_gradt_axpby(d, u, inv_h, nullptr, 0.0, out, s);
 }
 
-int helm_zchunks(Dims d) { return div_up(d.nz + 1, ZH); }
-
-int64_t helm_fp32_size(Dims d) {
-  const FaceGeom32 p = make_face_geom32(d);
-  return p.off[2] + p.sz[2] * p.n[2][2];
-}
-
-// x-blocks cover the nx first points of every row (a multiple of 4 when
-// rounded up); for u_x the remaining point x = nx is a wall face, never
-// written and kept 0 since the arrays were cleared at creation
-dim3 helm_v4_grid(Dims d) {
-  return dim3(div_up(div_up(d.nx, 4), 32), div_up(d.ny + 1, HVY), 3 * helm_zchunks(d));
-}
-
-void launch_helm_cheb(Dims d, const float* e, const float* eo, float* r32, float* rlo,
-                      const double* r64, double rs, float a, float nu_h2, float alpha, float beta,
-                      float* en, double* u, double us, int mode, cudaStream_t s, int flags,
-                      const float* pe, double ps) {
-  const FaceGeom32 p = make_face_geom32(d);
-  const float rs_hi = (float)rs, rs_lo = (float)(rs - (double)rs_hi);
-  count_launch();
-  const FaceGeom g = make_face_geom(d);
-  const int zch = helm_zchunks(d);
-  if (mode == 0)
-    launch_pdl(k_helm_cheb_v4<0>, helm_v4_grid(d), dim3(32, HVY), 0, s, g, p, zch, e, eo, r32,
-               rlo, r64, rs_hi, rs_lo, a, nu_h2, alpha, beta, en, u, us, pe, ps, flags);
-  else if (mode == 1)
-    launch_pdl(k_helm_cheb_v4<1>, helm_v4_grid(d), dim3(32, HVY), 0, s, g, p, zch, e, eo, r32,
-               rlo, r64, rs_hi, rs_lo, a, nu_h2, alpha, beta, en, u, us, pe, ps, flags);
-  else
-    launch_pdl(k_helm_cheb_v4<2>, helm_v4_grid(d), dim3(32, HVY), 0, s, g, p, zch, e, eo, r32,
-               rlo, r64, rs_hi, rs_lo, a, nu_h2, alpha, beta, en, u, us, pe, ps, flags);
-}
-
-// u = ps pe on the interior faces, 0 on the wall faces (a predictor
-// correction kept in FP32 written to the FP64 iterate when no later
-// correction's last step does it)
-__global__ void __launch_bounds__(32 * HVY) k_helm_flush(FaceGeom g, FaceGeom32 p, int zchunks,
-                                                         const float* __restrict__ pe, double ps,
-                                                         double* __restrict__ u) {
-  const int c = blockIdx.z / zchunks;
-  const int zc = blockIdx.z - c * zchunks;
-  const int x0 = 4 * (blockIdx.x * 32 + threadIdx.x);
-  const int j = blockIdx.y * HVY + threadIdx.y;
-  const int n0 = sel3(c, p.n[0][0], p.n[1][0], p.n[2][0]);
-  const int n1 = sel3(c, p.n[0][1], p.n[1][1], p.n[2][1]);
-  const int n2 = sel3(c, p.n[0][2], p.n[1][2], p.n[2][2]);
-  const int z0 = zc * ZH;
-  if (z0 >= n2 || x0 >= n0 || j >= n1) return;
-  const int z1 = min(z0 + ZH, n2);
-  const int64_t sy = sel3(c, p.sy[0], p.sy[1], p.sy[2]), sz = sel3(c, p.sz[0], p.sz[1], p.sz[2]);
-  const int64_t sy64 = sel3(c, g.sy[0], g.sy[1], g.sy[2]);
-  const int64_t sz64 = sel3(c, g.sz[0], g.sz[1], g.sz[2]);
-  int64_t f = sel3(c, p.off[0], p.off[1], p.off[2]) + (int64_t)z0 * sz + (int64_t)j * sy + x0;
-  int64_t f64 = sel3(c, g.off[0], g.off[1], g.off[2]) + (int64_t)z0 * sz64 + (int64_t)j * sy64 + x0;
-  const bool wally = c == 1 && (j == 0 || j == n1 - 1);
-  for (int z = z0; z < z1; ++z, f += sz, f64 += sz64) {
-    const bool wallz = c == 2 && (z == 0 || z == n2 - 1);
-    const float4 v = *reinterpret_cast<const float4*>(pe + f);
-    const float vq[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (x0 + q >= n0) break;
-      const bool wallx = c == 0 && (x0 + q == 0 || x0 + q == n0 - 1);
-      u[f64 + q] = (wallx || wally || wallz) ? 0.0 : ps * f2d_exact(vq[q]);
-    }
-  }
-}
-
-void launch_helm_flush(Dims d, const float* pe, double ps, double* u, cudaStream_t s) {
-  count_launch();
-  k_helm_flush<<<helm_v4_grid(d), dim3(32, HVY), 0, s>>>(make_face_geom(d), make_face_geom32(d),
-                                                          helm_zchunks(d), pe, ps, u);
-}
-
-int64_t launch_helm_resid_ds(Dims d, const float* e, float* rhi, float* rlo, double a,
-                             double nu_h2, double* part, int stride, cudaStream_t s) {
-  const dim3 gr = helm_v4_grid(d);
-  const float a_hi = (float)a, a_lo = (float)(a - (double)a_hi);
-  const float n_hi = (float)nu_h2, n_lo = (float)(nu_h2 - (double)n_hi);
-  count_launch();
-  k_helm_resid_ds<<<gr, dim3(32, HVY), 0, s>>>(make_face_geom32(d), helm_zchunks(d), e, rhi, rlo,
-                                               a_hi, a_lo, n_hi, n_lo, part, stride);
-  return (int64_t)gr.x * gr.y * gr.z;
-}
-
 // dsf of an FP64 constant (host)
 dsf host_ds(double x) {
   const float hi = (float)x;
   return dsf{hi, (float)(x - (double)hi)};
+}
+
+int64_t helm_fp32_size(Dims d) {
+  const HelmGeom p = make_helm_geom(d);
+  return p.off[2] + 2 * p.cs[2];
+}
+
+// Launch shape for `groups` threads' worth of a row: LX (32, 16 or 8) threads
+// per row so that few of them lie past its end, and planes per thread so that
+// there are about eight blocks per SM, at most 8 (several waves of blocks).
+struct HelmShape {
+  int lx, zc, zch;
+  dim3 grid, block;
+};
+
+HelmShape helm_shape(Dims d, int groups) {
+  HelmShape h;
+  h.lx = 32;
+  for (int lx : {16, 8})
+    if (div_up(groups, lx) * lx < div_up(groups, h.lx) * h.lx) h.lx = lx;
+  const int gx = div_up(groups, h.lx), gy = div_up(d.ny + 1, kHelmThreads / h.lx);
+  h.zc = (int)std::min<int64_t>(8, std::max<int64_t>(1, (int64_t)gx * gy * 3 * (d.nz + 1) / (152 * 8)));
+  h.zch = div_up(d.nz + 1, h.zc);
+  h.grid = dim3(gx, gy, 3 * h.zch);
+  h.block = dim3(h.lx, kHelmThreads / h.lx);
+  return h;
+}
+
+// 1 / (a + (6 + g) nu), g = 0..3 ghosts, times f
+float4 helm_weights(double a, double nu_h2, double f) {
+  auto w = [&](int g) { return (float)(f / (a + (6 + g) * nu_h2)); };
+  return make_float4(w(0), w(1), w(2), w(3));
+}
+
+void launch_helm_start(Dims d, const double* r64, float scale, double a, double nu_h2, float* rhi,
+                       float* rlo, float* e, cudaStream_t s) {
+  const HelmShape h = helm_shape(d, 2 * div_up(d.nx, 2));
+  count_launch();
+  k_helm_start<<<h.grid, h.block, 0, s>>>(make_face_geom(d), make_helm_geom(d), h.zc, h.zch, r64,
+                                          scale, helm_weights(a, nu_h2, 1.0), rhi, rlo, e);
+}
+
+void launch_helm_half(Dims d, int col, float* e, const float* r, double a, double nu_h2,
+                      double omega, bool old_zero, cudaStream_t s) {
+  const HelmShape h = helm_shape(d, div_up(d.nx, 8));
+  count_launch();
+  const bool full = d.nx % 8 == 0;
+  const auto k32 = full ? k_helm_half<32, true> : k_helm_half<32, false>;
+  const auto k16 = full ? k_helm_half<16, true> : k_helm_half<16, false>;
+  const auto k8 = full ? k_helm_half<8, true> : k_helm_half<8, false>;
+  launch_pdl(h.lx == 32 ? k32 : (h.lx == 16 ? k16 : k8), h.grid, h.block, 0, s, make_helm_geom(d),
+             h.zc, h.zch, col, e, r, (float)nu_h2, helm_weights(a, nu_h2, omega),
+             (float)(1.0 - omega), old_zero ? 1 : 0);
+}
+
+int64_t launch_helm_resid(Dims d, const float* e, float* rhi, float* rlo, double a, double nu_h2,
+                          float* en, double* part, cudaStream_t s) {
+  const HelmShape h = helm_shape(d, div_up(d.nx, 4));
+  const auto k = h.lx == 32 ? k_helm_resid<32> : (h.lx == 16 ? k_helm_resid<16> : k_helm_resid<8>);
+  count_launch();
+  k<<<h.grid, h.block, 0, s>>>(make_helm_geom(d), h.zc, h.zch, e, rhi, rlo, host_ds(a),
+                               host_ds(nu_h2), helm_weights(a, nu_h2, 1.0), en, part);
+  return (int64_t)h.grid.x * h.grid.y * h.grid.z;
+}
+
+void launch_helm_flush(Dims d, const float* e, const float* pe, int k, bool add, double* u,
+                       cudaStream_t s) {
+  const HelmShape h = helm_shape(d, 2 * div_up(d.nx, 2));
+  count_launch();
+  if (add)
+    k_helm_flush<true><<<h.grid, h.block, 0, s>>>(make_face_geom(d), make_helm_geom(d), h.zc,
+                                                  h.zch, e, pe, k, u);
+  else
+    k_helm_flush<false><<<h.grid, h.block, 0, s>>>(make_face_geom(d), make_helm_geom(d), h.zc,
+                                                   h.zch, e, pe, k, u);
 }
 
 void launch_predictor_rhs_adv(Dims d, const double* u_n, const double* u_nm1, const double* p_n,
