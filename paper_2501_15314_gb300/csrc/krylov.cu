@@ -7,14 +7,15 @@
 // (one FP32 V-cycle) is not an exact fixed linear map, and it measures the
 // unpreconditioned residual directly.
 //
-// Reductions are two-stage with a fixed grid (kRedBlocks blocks, fixed-order
-// tree inside each block, then one fixed-order tree per output): results are
-// bitwise reproducible run to run.
+// Reductions are two-stage with a grid set by the length (red_blocks blocks,
+// fixed-order tree inside each block, then one fixed-order tree per output):
+// results are bitwise reproducible run to run.
 #include <cmath>
 #include <vector>
 
 #include "ds.cuh"
 #include "ibm_internal.cuh"
+#include "reduce.cuh"
 
 namespace ibm {
 
@@ -34,20 +35,10 @@ __device__ __forceinline__ T warp_sum(T v) {
 // writes part[blockIdx.x * kOutStride + q].
 template <int NQ>
 __device__ __forceinline__ void block_reduce_store(double (&acc)[NQ], int nq, double* part) {
-  __shared__ double sh[RT / 32][NQ];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    const double v = warp_sum(acc[q]);
-    if (lane == 0) sh[wid][q] = v;
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < nq; q += RT) {
-    double s = 0.0;
-#pragma unroll
-    for (int w = 0; w < RT / 32; ++w) s += sh[w][q];
-    part[(int64_t)blockIdx.x * kOutStride + q] = s;
-  }
+  block_totals<NQ, RT / 32>(
+      acc, nq, part + (int64_t)blockIdx.x * kOutStride, [](double x, double y) { return x + y; },
+      [](double x, int o) { return __shfl_xor_sync(0xffffffffu, x, o); },
+      [](double x) { return x; });
 }
 
 // part[b][q] = sum over this block's elements of w_i * V_q[i], q < nq <= NQ
@@ -203,15 +194,16 @@ __global__ void k_add_scalar(double* __restrict__ x, int64_t n, const double* __
 #define IBM_NQ_DISPATCH(nq, KERNEL, ...)                          \
   do {                                                            \
     count_launch();                                               \
-    if ((nq) <= 2) KERNEL<2><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__);        \
-    else if ((nq) <= 4) KERNEL<4><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__);   \
-    else if ((nq) <= 8) KERNEL<8><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__);   \
-    else if ((nq) <= 12) KERNEL<12><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__); \
-    else if ((nq) <= 16) KERNEL<16><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__); \
-    else if ((nq) <= 24) KERNEL<24><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__); \
-    else if ((nq) <= 32) KERNEL<32><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__); \
-    else if ((nq) <= 48) KERNEL<48><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__); \
-    else KERNEL<kMaxRestart + 1><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__);    \
+    const int nb_ = red_blocks(n);                                \
+    if ((nq) <= 2) KERNEL<2><<<nb_, RT, 0, s>>>(__VA_ARGS__);        \
+    else if ((nq) <= 4) KERNEL<4><<<nb_, RT, 0, s>>>(__VA_ARGS__);   \
+    else if ((nq) <= 8) KERNEL<8><<<nb_, RT, 0, s>>>(__VA_ARGS__);   \
+    else if ((nq) <= 12) KERNEL<12><<<nb_, RT, 0, s>>>(__VA_ARGS__); \
+    else if ((nq) <= 16) KERNEL<16><<<nb_, RT, 0, s>>>(__VA_ARGS__); \
+    else if ((nq) <= 24) KERNEL<24><<<nb_, RT, 0, s>>>(__VA_ARGS__); \
+    else if ((nq) <= 32) KERNEL<32><<<nb_, RT, 0, s>>>(__VA_ARGS__); \
+    else if ((nq) <= 48) KERNEL<48><<<nb_, RT, 0, s>>>(__VA_ARGS__); \
+    else KERNEL<kMaxRestart + 1><<<nb_, RT, 0, s>>>(__VA_ARGS__);    \
   } while (0)
 
 }  // namespace
@@ -221,14 +213,14 @@ void launch_multidot(const double* w, const double* V, int64_t ld, int nq, int64
                      double* quot, double* hout) {
   IBM_NQ_DISPATCH(nq, k_multidot, w, V, ld, nq, n, part);
   count_launch();
-  k_final_reduce<<<nq, RT, 0, s>>>(part, kRedBlocks, out, div, quot, hout);
+  k_final_reduce<<<nq, RT, 0, s>>>(part, red_blocks(n), out, div, quot, hout);
 }
 
 void launch_axpy_norm(double* w, const double* V, int64_t ld, int nq, const double* coef,
                       int64_t n, double* part, double* out, cudaStream_t s, double* hout) {
   IBM_NQ_DISPATCH(nq, k_axpy_norm, w, V, ld, nq, coef, n, part);
   count_launch();
-  k_final_reduce<<<1, RT, 0, s>>>(part, kRedBlocks, out, nullptr, nullptr, hout);
+  k_final_reduce<<<1, RT, 0, s>>>(part, red_blocks(n), out, nullptr, nullptr, hout);
 }
 
 void launch_final_reduce(const double* part, int nb, double* out, cudaStream_t s,
@@ -240,17 +232,17 @@ void launch_final_reduce(const double* part, int nb, double* out, cudaStream_t s
 void launch_dot(const double* a, const double* b, int64_t n, double* part, double* out,
                 cudaStream_t s, double* hout) {
   count_launch();
-  k_dot<<<kRedBlocks, RT, 0, s>>>(a, b, n, part);
+  k_dot<<<red_blocks(n), RT, 0, s>>>(a, b, n, part);
   count_launch();
-  k_final_reduce<<<1, RT, 0, s>>>(part, kRedBlocks, out, nullptr, nullptr, hout);
+  k_final_reduce<<<1, RT, 0, s>>>(part, red_blocks(n), out, nullptr, nullptr, hout);
 }
 
 void launch_norm2_lead(const double* x, int64_t n, double* part, double* out, cudaStream_t s,
                        double* hout) {
   count_launch();
-  k_norm2_lead<<<kRedBlocks, RT, 0, s>>>(x, n, part);
+  k_norm2_lead<<<red_blocks(n), RT, 0, s>>>(x, n, part);
   count_launch();
-  k_final_reduce<<<1, RT, 0, s>>>(part, kRedBlocks, out, nullptr, nullptr, hout);
+  k_final_reduce<<<1, RT, 0, s>>>(part, red_blocks(n), out, nullptr, nullptr, hout);
 }
 
 namespace {

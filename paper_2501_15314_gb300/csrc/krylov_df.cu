@@ -18,6 +18,7 @@
 
 #include "ds.cuh"
 #include "ibm_internal.cuh"
+#include "reduce.cuh"
 
 namespace ibm {
 
@@ -31,34 +32,18 @@ __device__ __forceinline__ dsf d_to_ds(double x) {
   const float hi = (float)x;
   return {hi, (float)(x - (double)hi)};
 }
-__device__ __forceinline__ dsf ds_shfl_down(dsf a, int o) {
-  return {__shfl_down_sync(kFull, a.hi, o), __shfl_down_sync(kFull, a.lo, o)};
+__device__ __forceinline__ dsf ds_shfl_xor(dsf a, int o) {
+  return {__shfl_xor_sync(kFull, a.hi, o), __shfl_xor_sync(kFull, a.lo, o)};
 }
 
-// Reduces NQ double-single values across the block (warp shuffles, then the
-// warps in order) and stores the block sums as FP64 in part[block][q].
+// Reduces NQ double-single values across the block and stores the block sums
+// as FP64 in part[block][q].
 template <int NQ>
 __device__ __forceinline__ void block_reduce_ds(dsf (&acc)[NQ], int nq, double* part) {
-  __shared__ float sh_hi[RT / 32][NQ];
-  __shared__ float sh_lo[RT / 32][NQ];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    dsf v = acc[q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = ds_add(v, ds_shfl_down(v, o));
-    if (lane == 0) {
-      sh_hi[wid][q] = v.hi;
-      sh_lo[wid][q] = v.lo;
-    }
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < nq; q += RT) {
-    double s = 0.0;
-#pragma unroll
-    for (int w = 0; w < RT / 32; ++w) s += (double)sh_hi[w][q] + (double)sh_lo[w][q];
-    part[(int64_t)blockIdx.x * kOutStride + q] = s;
-  }
+  block_totals<NQ, RT / 32>(
+      acc, nq, part + (int64_t)blockIdx.x * kOutStride, [](dsf x, dsf y) { return ds_add(x, y); },
+      [](dsf x, int o) { return ds_shfl_xor(x, o); },
+      [](dsf x) { return (double)x.hi + (double)x.lo; });
 }
 
 // hi/lo split of an FP64 vector into interleaved pairs; the leading parts
@@ -456,10 +441,9 @@ __global__ void __launch_bounds__(RT) k_axpy_norm_sp(float* __restrict__ w,
 // 4 and nq <= 16.  Each element is accumulated exactly as in the scalar
 // kernels; only the order of the additions within a thread differs.
 template <int NQ>
-__global__ void __launch_bounds__(RT) k_multidot_sp4(const float4* __restrict__ w,
-                                                     const float4* __restrict__ V, int64_t ld4,
-                                                     int nq, int64_t n4,
-                                                     double* __restrict__ part) {
+__global__ void __launch_bounds__(RT, NQ <= 2 ? 8 : (NQ <= 4 ? 5 : (NQ <= 8 ? 3 : 2)))
+    k_multidot_sp4(const float4* __restrict__ w, const float4* __restrict__ V, int64_t ld4, int nq,
+                   int64_t n4, double* __restrict__ part) {
   pdl_wait();
   pdl_trigger();
   Comp acc[NQ];
@@ -552,22 +536,23 @@ __global__ void k_round_f32(const double* __restrict__ x, float* __restrict__ v,
 #define IBM_NQ_DISPATCH_DS(nq, KERNEL, ...)                                 \
   do {                                                                      \
     count_launch();                                                         \
-    if ((nq) <= 2) KERNEL<2><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__);        \
-    else if ((nq) <= 4) KERNEL<4><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__);   \
-    else if ((nq) <= 8) KERNEL<8><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__);   \
-    else if ((nq) <= 12) KERNEL<12><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__); \
-    else if ((nq) <= 16) KERNEL<16><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__); \
-    else if ((nq) <= 24) KERNEL<24><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__); \
-    else if ((nq) <= 32) KERNEL<32><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__); \
-    else if ((nq) <= 48) KERNEL<48><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__); \
-    else KERNEL<kMaxRestart + 1><<<kRedBlocks, RT, 0, s>>>(__VA_ARGS__);    \
+    const int nb_ = red_blocks(m);                                          \
+    if ((nq) <= 2) KERNEL<2><<<nb_, RT, 0, s>>>(__VA_ARGS__);        \
+    else if ((nq) <= 4) KERNEL<4><<<nb_, RT, 0, s>>>(__VA_ARGS__);   \
+    else if ((nq) <= 8) KERNEL<8><<<nb_, RT, 0, s>>>(__VA_ARGS__);   \
+    else if ((nq) <= 12) KERNEL<12><<<nb_, RT, 0, s>>>(__VA_ARGS__); \
+    else if ((nq) <= 16) KERNEL<16><<<nb_, RT, 0, s>>>(__VA_ARGS__); \
+    else if ((nq) <= 24) KERNEL<24><<<nb_, RT, 0, s>>>(__VA_ARGS__); \
+    else if ((nq) <= 32) KERNEL<32><<<nb_, RT, 0, s>>>(__VA_ARGS__); \
+    else if ((nq) <= 48) KERNEL<48><<<nb_, RT, 0, s>>>(__VA_ARGS__); \
+    else KERNEL<kMaxRestart + 1><<<nb_, RT, 0, s>>>(__VA_ARGS__);    \
   } while (0)
 
 // the float4 FP32 kernels, for nq <= 16
 #define IBM_NQ_DISPATCH_SP4(nq, KERNEL, ...)                                       \
   do {                                                                             \
     count_launch();                                                                \
-    const dim3 g_(kRedBlocks), b_(RT);                                             \
+    const dim3 g_(red_blocks(m / 4)), b_(RT);                                      \
     if ((nq) <= 2) launch_pdl(KERNEL<2>, g_, b_, 0, s, __VA_ARGS__);               \
     else if ((nq) <= 4) launch_pdl(KERNEL<4>, g_, b_, 0, s, __VA_ARGS__);          \
     else if ((nq) <= 8) launch_pdl(KERNEL<8>, g_, b_, 0, s, __VA_ARGS__);          \
@@ -965,6 +950,7 @@ ibm_status fgmres_solve_ds(ibm_ctx* c, const double* b, double* x, const ibm_sol
           IBM_OK)
         return sv;
       const int nq = jj + 1;
+      const int nb = red_blocks(vec4 && nq <= 16 ? m / 4 : m);
       ph = prof_begin(c, IBM_PROF_MULTIDOT);
       if (vec4 && nq <= 16)
         IBM_NQ_DISPATCH_SP4(nq, k_multidot_sp4, reinterpret_cast<const float4*>(w1),
@@ -974,7 +960,7 @@ ibm_status fgmres_solve_ds(ibm_ctx* c, const double* b, double* x, const ibm_sol
       else
         IBM_NQ_DISPATCH_DS(nq, k_multidot_ds, w, V2, m, nq, m, part);
       count_launch();
-      launch_pdl(k_final_reduce_ds, dim3(nq), dim3(RT), 0, s, (const double*)part, kRedBlocks,
+      launch_pdl(k_final_reduce_ds, dim3(nq), dim3(RT), 0, s, (const double*)part, nb,
                  raw, (const double*)nrm2, coef, coef_ds,
                  graph ? nullptr : hmirror(c, hr + (2 + (jj & 1)) * kOutStride));
       prof_end(c, ph, (single ? 4.0 : 8.0) * (nq + 1) * (double)m);
@@ -987,7 +973,7 @@ ibm_status fgmres_solve_ds(ibm_ctx* c, const double* b, double* x, const ibm_sol
       else
         IBM_NQ_DISPATCH_DS(nq, k_axpy_norm_ds, w, V2, m, nq, coef_ds, m, part, vin);
       count_launch();
-      launch_pdl(k_final_reduce_ds, dim3(1), dim3(RT), 0, s, (const double*)part, kRedBlocks,
+      launch_pdl(k_final_reduce_ds, dim3(1), dim3(RT), 0, s, (const double*)part, nb,
                  nrm2 + jj + 1, (const double*)nullptr, (double*)nullptr, (float2*)nullptr,
                  graph ? nullptr : hmirror(c, hr + 4 * kOutStride + jj + 1));
       // V_0..V_j and w read, w written (and its leading parts for the pair form)
