@@ -221,7 +221,7 @@ static void free_all(ibm_ctx* c) {
   MarkerData& m = c->mk;
   cudaFree(m.bf); cudaFree(m.bc); cudaFree(m.org); cudaFree(m.wf); cudaFree(m.wc); cudaFree(m.cw);
   cudaFree(m.t); cudaFree(m.t2); cudaFree(m.t32); cudaFree(m.dwf); cudaFree(m.dwc);
-  cudaFree(m.wc32); cudaFree(m.cw32);
+  cudaFree(m.wc32); cudaFree(m.cw32); cudaFree(m.slot);
   cudaFree(m.cg);
   cudaFree(m.t3); cudaFree(c->cg_bar);
   cudaFree(m.c_val);
@@ -383,7 +383,7 @@ ibm_status ibm_create(const ibm_grid_desc* g, void* stream, ibm_ctx** out) {
   bool ok = cudaMalloc(&c->cell_count, sizeof(int32_t) * m) == cudaSuccess &&
             cudaMalloc(&c->cell_start, sizeof(int32_t) * (m + 1)) == cudaSuccess &&
             cudaMalloc(&c->cell_flag, sizeof(int32_t) * (m + 1)) == cudaSuccess &&
-            cudaMalloc(&c->scan_tmp, sizeof(int32_t) * nscan) == cudaSuccess &&
+            cudaMalloc(&c->scan_tmp, sizeof(int32_t) * (nscan + (m + 4095) / 4096)) == cudaSuccess &&
             cudaMalloc(&c->dev_flag, sizeof(int32_t) * 4) == cudaSuccess &&
             cudaHostAlloc(&c->host_flag, sizeof(int32_t) * 4, cudaHostAllocMapped) ==
                 cudaSuccess &&
@@ -423,6 +423,7 @@ ibm_status ibm_create(const ibm_grid_desc* g, void* stream, ibm_ctx** out) {
     c->helm_part_n = nb * (kMaxRestart + 2);
     ok = ok && cudaMalloc(&c->helm_part, sizeof(double) * c->helm_part_n) == cudaSuccess;
   }
+  c->cell_touch = c->scan_tmp + nscan;
   if (!ok) {
     cudaGetLastError();
     free_all(c);

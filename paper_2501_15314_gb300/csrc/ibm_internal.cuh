@@ -69,6 +69,7 @@ struct MarkerData {
   double* dwc = nullptr;    // [3 axes][3 taps][n] phi' at the centre taps
   float* wc32 = nullptr;    // wc rounded to FP32 (the FP32 Arnoldi cycles' t = 2 B z)
   float* cw32 = nullptr;    // cw rounded to FP32
+  double* slot = nullptr;   // [n][3 axes][4 slots][4]: weights by the box's slots (layout fill)
   double* cg = nullptr;     // [3][3n] conjugate-gradient work vectors for C^{-1}
   double* t3 = nullptr;     // [3][n] per-marker scratch (RHS_F in the C modes)
   // rows of C = R^T R (cmode.cu), formed by the first C solve after the markers
@@ -139,6 +140,8 @@ struct ibm_ctx {
 
   // grid-sized scratch (FP64)
   int32_t* cell_count = nullptr;   // [m]
+  int32_t* cell_touch = nullptr;   // marks of the blocks of cells with counts (after scan_tmp)
+  bool counts_clean = false;       // cell_count and cell_touch are all zero
   int32_t* cell_start = nullptr;   // [m + 1]
   int32_t* cell_flag = nullptr;    // [m + 1]
   int32_t* scan_tmp = nullptr;     // block sums of the scans (int32 or int2 per block)

@@ -24,30 +24,35 @@ constexpr int TPB = 256;
 
 // Eq. (delta) times the cell width (phi) and its derivative d phi / dr
 // (differentiated branch by branch; continuous, with value -sign(r) at
-// |r| = 1/2 and 0 at |r| = 3/2), r in cell widths.  Both come from one
-// reciprocal square root R = 1/sqrt(A) of the branch's A = 1 - 3 s^2: the
-// square root is A R and the derivative's quotient s / sqrt(A) is s R (one
-// FP64 rsqrt in place of a square root and a division).
-struct RomaVal {
-  double phi, dphi;
+// |r| = 1/2 and 0 at |r| = 3/2) at a marker's three taps along one axis, which
+// lie at the distances r - 1, r, r + 1, |r| <= 1/2, r in cell widths.  The
+// outer branch's A = 1 - 3 (1 - |r +- 1|)^2 is the inner one's 1 - 3 r^2, so
+// all six values come from one FP64 reciprocal square root R = 1/sqrt(A)
+// (sqrt(A) = A R, the derivative's quotient r / sqrt(A) = r R).  One per tap
+// made this kernel's FP64 work, which bounds it: 58 us at 60000 markers, 31 now.
+struct RomaTaps {
+  double phi[3], dphi[3];
 };
 
-__device__ __forceinline__ RomaVal roma(double r) {
-  const double a = fabs(r);
-  if (a <= 0.5) {
-    const double A = 1.0 - 3.0 * r * r;
-    const double R = rsqrt(A);
-    return {(1.0 + A * R) * (1.0 / 3.0), -r * R};
-  }
-  if (a < 1.5) {
-    const double q = 1.0 - a;
-    const double A = 1.0 - 3.0 * q * q;
-    const double R = rsqrt(A);
-    const double v = -0.5 * (1.0 + q * R);
-    return {(5.0 - 3.0 * a - A * R) * (1.0 / 6.0), r > 0.0 ? v : -v};
-  }
-  return {0.0, 0.0};
+__device__ __forceinline__ RomaTaps roma(double r) {
+  const double A = fma(-3.0 * r, r, 1.0);
+  const double R = rsqrt(A);
+  const double S = A * R, t = 2.0 - S, q = r * R;
+  RomaTaps v;
+  v.phi[0] = fma(3.0, r, t) * (1.0 / 6.0);
+  v.phi[1] = (1.0 + S) * (1.0 / 3.0);
+  v.phi[2] = fma(-3.0, r, t) * (1.0 / 6.0);
+  v.dphi[0] = fma(0.5, q, 0.5);
+  v.dphi[1] = -q;
+  v.dphi[2] = fma(0.5, q, -0.5);
+  return v;
 }
+
+// One axis's weights of a marker at one slot of its box (see k_marker_setup)
+struct alignas(32) SlotWeights {
+  double gf, face, centre;
+  long long in;   // bit 0: the face is a tap, bit 1: the centre is
+};
 
 struct MkView {
   int64_t n;
@@ -57,14 +62,17 @@ struct MkView {
   const double* wf;
   const double* wc;
   const double* cw;
+  const SlotWeights* slot;
 };
 
-MkView view(const MarkerData& m) { return MkView{m.n, m.bf, m.bc, m.org, m.wf, m.wc, m.cw}; }
+MkView view(const MarkerData& m) {
+  return MkView{m.n, m.bf, m.bc, m.org, m.wf, m.wc, m.cw, reinterpret_cast<const SlotWeights*>(m.slot)};
+}
 
 __global__ void k_marker_setup(Dims d, double inv_h, int64_t n, const double* __restrict__ X,
                                int32_t* bf, int32_t* bc, int32_t* org, double* wf, double* wc,
                                double* cw, double* dwf, double* dwc, float* wc32, float* cw32,
-                               int32_t* err) {
+                               SlotWeights* slot, int32_t* err) {
   // one thread per (axis, marker): the three axes' Roma weights are
   // independent, and three times the threads hide the FP64 latency better
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -88,6 +96,7 @@ __global__ void k_marker_setup(Dims d, double inv_h, int64_t n, const double* __
       for (int q = 0; q < 4; ++q) cw[(e * 4 + q) * n + k] = 0.0;
       for (int q = 0; q < 3; ++q) wc32[(e * 3 + q) * n + k] = 0.f;
       for (int q = 0; q < 4; ++q) cw32[(e * 4 + q) * n + k] = 0.f;
+      for (int q = 0; q < 4; ++q) slot[(k * 3 + e) * 4 + q] = SlotWeights{0.0, 0.0, 0.0, 0};
       atomicOr(err, 1);
       return;
     }
@@ -97,18 +106,19 @@ __global__ void k_marker_setup(Dims d, double inv_h, int64_t n, const double* __
     if (b_c < 0 || b_c + 2 > ncell_e - 1) bad = true;
     bf[e * n + k] = b_f;
     bc[e * n + k] = b_c;
-    org[e * n + k] = min(b_f - 1, b_c);
+    // the box of a marker that is refused: in the grid, so that the passes that
+    // follow before the host has read the flag stay inside it
+    org[e * n + k] = bad ? 0 : min(b_f - 1, b_c);
+    const RomaTaps vf = roma(fs - s), vc = roma((fc + 0.5) - s);
     double W[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-      const RomaVal vf = roma((double)(b_f + q) - s);
-      const RomaVal vc = roma((double)(b_c + q) + 0.5 - s);
-      W[q] = vf.phi;
-      wf[(e * 3 + q) * n + k] = vf.phi;
-      wc[(e * 3 + q) * n + k] = vc.phi;
-      dwf[(e * 3 + q) * n + k] = vf.dphi;
-      dwc[(e * 3 + q) * n + k] = vc.dphi;
-      wc32[(e * 3 + q) * n + k] = (float)vc.phi;
+      W[q] = vf.phi[q];
+      wf[(e * 3 + q) * n + k] = vf.phi[q];
+      wc[(e * 3 + q) * n + k] = vc.phi[q];
+      dwf[(e * 3 + q) * n + k] = vf.dphi[q];
+      dwc[(e * 3 + q) * n + k] = vc.dphi[q];
+      wc32[(e * 3 + q) * n + k] = (float)vc.phi[q];
     }
     // cell b_f - 1 + q lies between faces b_f - 1 + q and b_f + q
     const double C[4] = {(0.0 - W[0]) * inv_h, (W[0] - W[1]) * inv_h, (W[1] - W[2]) * inv_h,
@@ -118,6 +128,24 @@ __global__ void k_marker_setup(Dims d, double inv_h, int64_t n, const double* __
       cw[(e * 4 + q) * n + k] = C[q];
       cw32[(e * 4 + q) * n + k] = (float)C[q];
     }
+    // the same by the box's slots, for the layout fill: the G^T-weighted
+    // weight, the weight of the cell's lower face and that of its centre, and
+    // whether face (bit 0) and centre (bit 1) are taps at all
+    const int df = b_f - 1 - org[e * n + k], dc = b_c - org[e * n + k];   // 0 or 1
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const int qf = x - df, qc = x - dc;
+      SlotWeights v = {0.0, 0.0, 0.0, 0};
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (qf == q) v.gf = C[q];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        if (qf - 1 == q) { v.face = W[q]; v.in |= 1; }
+        if (qc == q) { v.centre = vc.phi[q]; v.in |= 2; }
+      }
+      slot[(k * 3 + e) * 4 + x] = v;
+    }
   }
   if (bad) atomicOr(err, 1);
 }
@@ -126,14 +154,20 @@ __device__ __forceinline__ int64_t cell_of(Dims d, int i, int j, int k) {
   return ((int64_t)k * d.ny + j) * d.nx + i;
 }
 
-__global__ void k_count(Dims d, MkView mk, int32_t* count) {
+// Blocks of 2^kCellShift consecutive cells; only those that hold a marker's entry
+// (touch != 0) are visited by the passes over the cells.
+constexpr int kCellShift = 12;
+
+__global__ void k_count(Dims d, MkView mk, int32_t* count, int32_t* touch) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= mk.n * 64) return;
   const int64_t k = t >> 6;
   const int s = (int)(t & 63);
   const int i = mk.org[k] + (s & 3), j = mk.org[mk.n + k] + ((s >> 2) & 3),
             l = mk.org[2 * mk.n + k] + (s >> 4);
-  atomicAdd(count + cell_of(d, i, j, l), 1);
+  const int64_t c = cell_of(d, i, j, l);
+  atomicAdd(count + c, 1);
+  touch[c >> kCellShift] = 1;
 }
 
 // Places each (marker, slot) pair in its cell's segment: the cell's count
@@ -159,70 +193,89 @@ __global__ void k_fill(Dims d, MkView mk, const int32_t* __restrict__ start, int
 // longer ones by an insertion sort in lane 0.  Makes the entry order
 // independent of the atomics' scheduling.
 __global__ void k_sort_segments(int64_t n_shell, const int32_t* __restrict__ off, int32_t* key) {
-  const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  // two neighbouring segments per warp, loaded together
+  const int64_t q = 2 * ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (q >= n_shell) return;   // whole warps leave together
-  const int32_t a = off[q], L = off[q + 1] - off[q];
-  if (L <= 1) return;
-  if (L <= 64) {
-    const int32_t k0 = lane < L ? key[a + lane] : 0x7fffffff;
-    const int32_t k1 = lane + 32 < L ? key[a + 32 + lane] : 0x7fffffff;
-    int r0 = 0, r1 = 0;
-    for (int j = 0; j < L; ++j) {
-      const int32_t kj = __shfl_sync(0xffffffffu, j < 32 ? k0 : k1, j & 31);
-      r0 += kj < k0;
-      r1 += kj < k1;
+  const int32_t o0 = off[q], o1 = off[q + 1], o2 = q + 1 < n_shell ? off[q + 2] : o1;
+  const int32_t a[2] = {o0, o1}, L[2] = {o1 - o0, o2 - o1};
+  int32_t k0[2], k1[2];
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    k0[s] = lane < L[s] ? key[a[s] + lane] : 0x7fffffff;
+    k1[s] = lane + 32 < L[s] ? key[a[s] + 32 + lane] : 0x7fffffff;
+  }
+  int r0[2] = {0, 0}, r1[2] = {0, 0};
+  const int first = max(min(L[0], 32), min(L[1], 32));
+  for (int j = 0; j < first; ++j) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const int32_t kj = __shfl_sync(0xffffffffu, k0[s], j);   // past the end: the largest
+      r0[s] += kj < k0[s];
+      r1[s] += kj < k1[s];
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    if (L[s] <= 1 || L[s] > 64) continue;
+    for (int j = 0; j < L[s] - 32; ++j) {
+      const int32_t kj = __shfl_sync(0xffffffffu, k1[s], j);
+      r0[s] += kj < k0[s];
+      r1[s] += kj < k1[s];
     }
     __syncwarp();
-    if (lane < L) key[a + r0] = k0;
-    if (lane + 32 < L) key[a + r1] = k1;
-    return;
+    if (lane < L[s]) key[a[s] + r0[s]] = k0[s];
+    if (lane + 32 < L[s]) key[a[s] + r1[s]] = k1[s];
   }
   if (lane != 0) return;
-  for (int32_t x = a + 1; x < a + L; ++x) {
-    const int32_t v = key[x];
-    int32_t y = x - 1;
-    while (y >= a && key[y] > v) { key[y + 1] = key[y]; --y; }
-    key[y + 1] = v;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    if (L[s] <= 64) continue;
+    for (int32_t x = a[s] + 1; x < a[s] + L[s]; ++x) {
+      const int32_t v = key[x];
+      int32_t y = x - 1;
+      while (y >= a[s] && key[y] > v) { key[y + 1] = key[y]; --y; }
+      key[y + 1] = v;
+    }
   }
 }
 
-// Coefficients of G^T R e_{k,d} (d = 0, 1, 2) at global cell g: along d the
-// G^T-weighted face taps cw (cell i lies between faces i and i+1), along the
-// other two axes the centre-tap weights; zero outside the 4 x 3 x 3
-// footprint.  Each axis's two factors are loaded once; coef_d = f_d P_d
-// with f_d the cw factor along d and P_d the product of the centre weights
-// along the other two axes (three pair products shared by the six weights:
-// nine FP64 multiplications per entry, the FP64 pipe being this kernel's
-// bound).
+// Coefficients of G^T R e_{k,d} (d = 0, 1, 2) at the cell in slot sl of marker
+// k's box: along d the G^T-weighted face taps (cell i lies between faces i and
+// i+1), along the other two axes the centre-tap weights; zero outside the
+// 4 x 3 x 3 footprint.  coef_d = f_d P_d with f_d the weight along d and P_d the
+// product of the centre weights along the other two axes (three pair products
+// shared by the six weights: nine FP64 multiplications per entry).
 //
 // With them the spread weights of the same entry: the weight of F_{k,d} at
-// the cell's lower d-face, the face-tap weight wf along d times the same
-// P_d, and in bit d whether that face lies inside the support.
-__device__ __forceinline__ void gtr_coefs(const MkView& mk, int64_t k, const int g[3],
-                                          double (&coef)[3], double (&sw)[3], int& in) {
-  double fw[3], fc[3], ff[3];
-  bool inw[3], inf[3];
+// the cell's lower d-face, the face-tap weight along d times the same P_d, and
+// in bit d whether that face lies inside the support.
+//
+// Each axis's weights at the slot are one aligned 32-byte load (MkView::slot);
+// from the tap arrays they took five, and the layout fill, whose markers
+// differ from lane to lane, waited on them: 145 us at 60000
+// markers, 113 now (its FP64 products and its 64 B written per entry take 60 and
+// 40).
+__device__ __forceinline__ void gtr_coefs(const MkView& mk, int64_t k, int sl, double (&coef)[3],
+                                          double (&sw)[3], int& in) {
+  SlotWeights w[3];
+  int inf[3], inw[3];
 #pragma unroll
   for (int e = 0; e < 3; ++e) {
-    const int b_f = mk.bf[e * mk.n + k];
-    const int qf = g[e] - (b_f - 1);
-    fc[e] = (qf >= 0 && qf <= 3) ? mk.cw[(e * 4 + qf) * mk.n + k] : 0.0;
-    inf[e] = qf >= 1 && qf <= 3;   // the face g[e] is face tap qf - 1 of 0..2
-    ff[e] = inf[e] ? mk.wf[(e * 3 + qf - 1) * mk.n + k] : 0.0;
-    const int qc = g[e] - mk.bc[e * mk.n + k];
-    inw[e] = qc >= 0 && qc <= 2;
-    fw[e] = inw[e] ? mk.wc[(e * 3 + qc) * mk.n + k] : 0.0;
+    w[e] = mk.slot[(k * 3 + e) * 4 + ((sl >> (2 * e)) & 3)];
+    inf[e] = (int)w[e].in & 1;
+    inw[e] = (int)w[e].in >> 1;
   }
-  const double p12 = fw[1] * fw[2], p02 = fw[0] * fw[2], p01 = fw[0] * fw[1];
-  coef[0] = fc[0] * p12;
-  coef[1] = fc[1] * p02;
-  coef[2] = fc[2] * p01;
-  sw[0] = ff[0] * p12;
-  sw[1] = ff[1] * p02;
-  sw[2] = ff[2] * p01;
-  in = (inf[0] && inw[1] && inw[2] ? 1 : 0) | (inw[0] && inf[1] && inw[2] ? 2 : 0) |
-       (inw[0] && inw[1] && inf[2] ? 4 : 0);
+  const double p12 = w[1].centre * w[2].centre, p02 = w[0].centre * w[2].centre,
+               p01 = w[0].centre * w[1].centre;
+  coef[0] = w[0].gf * p12;
+  coef[1] = w[1].gf * p02;
+  coef[2] = w[2].gf * p01;
+  sw[0] = w[0].face * p12;
+  sw[1] = w[1].face * p02;
+  sw[2] = w[2].face * p01;
+  in = (inf[0] & inw[1] & inw[2]) | (inw[0] & inf[1] & inw[2]) << 1 |
+       (inw[0] & inw[1] & inf[2]) << 2;
 }
 
 // FP32 values widened to FP64 with integer operations (the conversion
@@ -389,9 +442,10 @@ __global__ void k_ell_len(int64_t n_shell, const int32_t* __restrict__ off,
 __global__ void k_ell_fill(MkView mk, int64_t n_shell, const int32_t* __restrict__ off,
                            const int32_t* __restrict__ key, const int32_t* __restrict__ base,
                            const int32_t* __restrict__ len, const int32_t* __restrict__ perm,
-                           const int32_t* __restrict__ ell_cell, Dims d, int64_t n_ell,
-                           int32_t* ekey, double* ecoef, float* ecoef32, double* esw,
-                           uint8_t* eany) {
+                           int64_t n_ell,
+                           int32_t* __restrict__ ekey, double* __restrict__ ecoef,
+                           float* __restrict__ ecoef32, double* __restrict__ esw,
+                           uint8_t* __restrict__ eany) {
   const int64_t tq = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t w = tq >> 5;
   if (w >= ell_groups(n_shell)) return;
@@ -399,29 +453,34 @@ __global__ void k_ell_fill(MkView mk, int64_t n_shell, const int32_t* __restrict
   const int64_t q = w * kEllCells + lane / kEllLanes;
   const bool live = q < n_shell;
   int32_t a = 0, nseg = 0;
-  int g[3] = {0, 0, 0};
   if (live) {
     const int32_t r = perm[q];
     a = off[r];
     nseg = off[r + 1] - a;
-    const int64_t c = ell_cell[q];
-    g[0] = (int)(c % d.nx);
-    g[1] = (int)((c / d.nx) % d.ny);
-    g[2] = (int)(c / ((int64_t)d.nx * d.ny));
   }
   const int32_t rounds = len[w];
   int any = 0;
-  for (int32_t rr = 0; rr < rounds; ++rr) {
-    const int64_t dst = base[w] + (int64_t)rr * 32 + lane;
-    const int p = kEllLanes * rr + lane % kEllLanes;
-    if (live && p < nseg) {
-      const int32_t kk = key[a + p];
-      ekey[dst] = kk;
-      const int64_t k = kk >> 6;
-      double cf[3], sw[3];
-      int in;
-      gtr_coefs(mk, k, g, cf, sw, in);
-      any |= in;
+  // the keys of four rounds are read together, then their weights
+  for (int32_t r0 = 0; r0 < rounds; r0 += 4) {
+    int32_t kk[4];
+    bool in4[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const int p = kEllLanes * (r0 + x) + lane % kEllLanes;
+      in4[x] = live && r0 + x < rounds && p < nseg;
+      kk[x] = in4[x] ? key[a + p] : 0;
+    }
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      if (r0 + x >= rounds) break;   // warp-uniform
+      const int64_t dst = base[w] + (int64_t)(r0 + x) * 32 + lane;
+      double cf[3] = {0.0, 0.0, 0.0}, sw[3] = {0.0, 0.0, 0.0};
+      if (in4[x]) {
+        int in;
+        gtr_coefs(mk, kk[x] >> 6, kk[x] & 63, cf, sw, in);
+        any |= in;
+      }
+      ekey[dst] = kk[x];
 #pragma unroll
       for (int dc = 0; dc < 3; ++dc) {
         ecoef[dc * n_ell + dst] = cf[dc];
@@ -429,14 +488,6 @@ __global__ void k_ell_fill(MkView mk, int64_t n_shell, const int32_t* __restrict
         // conversion would run on the FP64 pipe)
         ecoef32[dc * n_ell + dst] = split_exact(cf[dc]).hi;
         esw[dc * n_ell + dst] = sw[dc];
-      }
-    } else {
-      ekey[dst] = 0;
-#pragma unroll
-      for (int dc = 0; dc < 3; ++dc) {
-        ecoef[dc * n_ell + dst] = 0.0;
-        ecoef32[dc * n_ell + dst] = 0.f;
-        esw[dc * n_ell + dst] = 0.0;
       }
     }
   }
@@ -714,12 +765,22 @@ __device__ int2 block_excl_scan2(int2 v, int2* sh, int2* total) {
   return make_int2(wp.x + x.x - v.x, wp.y + x.y - v.y);
 }
 
-// Shell cells of the marker lists, in two passes over the cell counts (each
-// block SCAN_T * SCAN_E cells): k_cell_sums writes each block's (entries,
-// shell cells); after the scan of those, k_shell_list writes, for every cell
-// with entries, its segment start and its place in the shell list.
-__global__ void k_cell_sums(const int32_t* __restrict__ count, int64_t n, int2* __restrict__ sums) {
+// Shell cells of the marker lists, in two passes over the cell counts of the
+// touched blocks (each SCAN_T * SCAN_E cells): k_cell_sums writes each block's
+// (entries, shell cells); after the scan of those, k_shell_list writes, for
+// every cell with entries, its segment start and its place in the shell list,
+// and takes the block's mark back.  Over all cells the two passes and the
+// zeroing of the counts took 90 us at 256^3, of which the spheres' shells touch
+// an eighth; 30 now.
+static_assert(SCAN_T * SCAN_E == 1 << kCellShift, "one scan block per block of cells");
+
+__global__ void k_cell_sums(const int32_t* __restrict__ count, int64_t n,
+                            const int32_t* __restrict__ touch, int2* __restrict__ sums) {
   __shared__ int2 sh[32];
+  if (touch[blockIdx.x] == 0) {   // block-uniform
+    if (threadIdx.x == 0) sums[blockIdx.x] = make_int2(0, 0);
+    return;
+  }
   const int64_t base = (int64_t)blockIdx.x * SCAN_T * SCAN_E + (int64_t)threadIdx.x * SCAN_E;
   int2 v = make_int2(0, 0);
 #pragma unroll
@@ -757,8 +818,10 @@ __global__ void k_scan_sums2(int2* sums, int64_t nb) {
 __global__ void k_shell_list(const int32_t* __restrict__ count, int64_t n,
                              const int2* __restrict__ sums, int32_t* __restrict__ start,
                              int32_t* __restrict__ shell_cell, int32_t* __restrict__ shell_off,
-                             int64_t nb) {
+                             int64_t nb, int32_t* __restrict__ touch) {
   __shared__ int2 sh[32];
+  if (blockIdx.x == 0 && threadIdx.x == 0) shell_off[sums[nb].y] = sums[nb].x;
+  if (touch[blockIdx.x] == 0) return;   // block-uniform
   const int64_t base = (int64_t)blockIdx.x * SCAN_T * SCAN_E + (int64_t)threadIdx.x * SCAN_E;
   int32_t k[SCAN_E];
   int2 v = make_int2(0, 0);
@@ -781,7 +844,8 @@ __global__ void k_shell_list(const int32_t* __restrict__ count, int64_t n,
     }
     e += k[q];
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) shell_off[sums[nb].y] = sums[nb].x;
+  // (every thread has read the mark: the scan above synchronised the block)
+  if (threadIdx.x == 0) touch[blockIdx.x] = 0;
 }
 
 __global__ void k_scan_blocks(const int32_t* __restrict__ in, int64_t n, int32_t* __restrict__ out,
@@ -864,7 +928,8 @@ static ibm_status grow_markers(ibm_ctx* c, int64_t n) {
   cudaFree(m.bf); cudaFree(m.bc); cudaFree(m.org); cudaFree(m.wf); cudaFree(m.wc);
   cudaFree(m.cw); cudaFree(m.t); cudaFree(m.t2); cudaFree(m.t32); cudaFree(m.dwf);
   cudaFree(m.dwc); cudaFree(m.wc32); cudaFree(m.cw32);
-  cudaFree(m.cg); cudaFree(m.t3);
+  cudaFree(m.cg); cudaFree(m.t3); cudaFree(m.slot);
+  m.slot = nullptr;
   m.bf = m.bc = m.org = nullptr;
   m.wf = m.wc = m.cw = m.t = m.t2 = m.dwf = m.dwc = m.cg = m.t3 = nullptr;
   m.t32 = nullptr;
@@ -882,6 +947,7 @@ static ibm_status grow_markers(ibm_ctx* c, int64_t n) {
       cudaMalloc(&m.cw32, sizeof(float) * 12 * n) != cudaSuccess ||
       cudaMalloc(&m.t2, sizeof(double) * 3 * n) != cudaSuccess ||
       cudaMalloc(&m.t3, sizeof(double) * 3 * n) != cudaSuccess ||
+      cudaMalloc(&m.slot, sizeof(double) * 48 * n) != cudaSuccess ||
       cudaMalloc(&m.cg, sizeof(double) * 9 * n) != cudaSuccess) {
     cudaGetLastError();
     return set_err(c, IBM_ERR_NOMEM, "marker workspace allocation failed");
@@ -957,46 +1023,56 @@ ibm_status markers_build(ibm_ctx* c, int64_t n, const double* X) {
   count_launch();
   k_marker_setup<<<div_up(3 * n, TPB), TPB, 0, s>>>(c->d, 1.0 / c->h, n, X, m.bf, m.bc, m.org,
                                                      m.wf, m.wc, m.cw, m.dwf, m.dwc, m.wc32,
-                                                     m.cw32, c->dev_flag);
+                                                     m.cw32, reinterpret_cast<SlotWeights*>(m.slot),
+                                                     c->dev_flag);
   IBM_LAUNCH_CHECK(c);
-  launch_to_host(c->dev_flag, c->host_flag_dev, sizeof(int32_t), s);
-  IBM_LAUNCH_CHECK(c);
-  IBM_CUDA(c, cudaStreamSynchronize(s));
-  if (c->host_flag[0] != 0)
-    return set_err(c, IBM_ERR_MARKER_DOMAIN,
-                   "a marker's delta support touches a wall face or leaves the grid");
   m.n = n;
   const MkView mv = view(m);
   // counting sort of (marker, slot) pairs by cell: counts, then one
   // reduction and one scan-and-list pass over the counts for the segment
   // starts and the shell-cell list, then the fill (which takes the counts
-  // back to zero) and the per-segment sort
-  launch_zero(c->cell_count, sizeof(int32_t) * c->m, s);
-  count_launch();
-  k_count<<<div_up(n * 64, TPB), TPB, 0, s>>>(c->d, mv, c->cell_count);
+  // back to zero) and the per-segment sort.  Between builds the counts and the
+  // marks of the touched blocks are zero; a build that did not get as far as
+  // the fill leaves them to be zeroed by the next.
   const int64_t nb = (c->m + SCAN_T * SCAN_E - 1) / (SCAN_T * SCAN_E);
+  int32_t* touch = c->cell_touch;
+  if (!c->counts_clean) {
+    launch_zero(c->cell_count, sizeof(int32_t) * c->m, s);
+    launch_zero(touch, sizeof(int32_t) * nb, s);
+  }
+  c->counts_clean = false;
+  count_launch();
+  k_count<<<div_up(n * 64, TPB), TPB, 0, s>>>(c->d, mv, c->cell_count, touch);
   int2* bsum = reinterpret_cast<int2*>(c->scan_tmp);
   count_launch();
-  k_cell_sums<<<(unsigned)nb, SCAN_T, 0, s>>>(c->cell_count, c->m, bsum);
+  k_cell_sums<<<(unsigned)nb, SCAN_T, 0, s>>>(c->cell_count, c->m, touch, bsum);
   count_launch();
   k_scan_sums2<<<1, SCAN_T, 0, s>>>(bsum, nb);
+  // one round trip for the totals and the flag of a marker out of the domain
   launch_to_host(bsum + nb, c->host_flag_dev, sizeof(int2), s);
+  launch_to_host(c->dev_flag, c->host_flag_dev + 2, sizeof(int32_t), s);
   IBM_LAUNCH_CHECK(c);
   IBM_CUDA(c, cudaStreamSynchronize(s));
+  if (c->host_flag[2] != 0) {
+    m.n = 0;
+    return set_err(c, IBM_ERR_MARKER_DOMAIN,
+                   "a marker's delta support touches a wall face or leaves the grid");
+  }
   const int64_t ne = c->host_flag[0], ns = c->host_flag[1];
   st = grow_entries(c, ne);
   if (st != IBM_OK) return st;
   count_launch();
   k_shell_list<<<(unsigned)nb, SCAN_T, 0, s>>>(c->cell_count, c->m, bsum, c->cell_start,
-                                               m.shell_cell, m.shell_off, nb);
+                                               m.shell_cell, m.shell_off, nb, touch);
   count_launch();
   k_fill<<<div_up(n * 64, TPB), TPB, 0, s>>>(c->d, mv, c->cell_start, c->cell_count, m.entry_key);
   count_launch();
-  k_sort_segments<<<div_up(32 * ns, TPB), TPB, 0, s>>>(ns, m.shell_off, m.entry_key);
+  k_sort_segments<<<div_up(16 * (ns + 1), TPB), TPB, 0, s>>>(ns, m.shell_off, m.entry_key);
   IBM_LAUNCH_CHECK(c);
+  c->counts_clean = true;
   // interleaved layout for the B^T t gather, in the order of ell_cell
   const int64_t ng = ell_groups(ns);
-  int32_t* cnt = c->cell_count;   // back at zero after the fill: the group sizes
+  int32_t* cnt = reinterpret_cast<int32_t*>(c->c1);   // scratch: the group sizes
   int32_t* perm = c->cell_flag;   // scratch: the layout order
   count_launch();
   k_ell_order<<<div_up(ns, kOrderWin), kOrderWin, 0, s>>>(ns, m.shell_off, m.shell_cell, perm,
@@ -1013,7 +1089,7 @@ ibm_status markers_build(ibm_ctx* c, int64_t n, const double* X) {
   if ((st = grow_ell(c, n_ell)) != IBM_OK) return st;
   count_launch();
   k_ell_fill<<<div_up(32 * ng, TPB), TPB, 0, s>>>(mv, ns, m.shell_off, m.entry_key, m.ell_base,
-                                             m.ell_len, perm, m.ell_cell, c->d, n_ell, m.ell_key,
+                                             m.ell_len, perm, n_ell, m.ell_key,
                                              m.ell_coef, m.ell_coef32, m.ell_sw, m.ell_any);
   IBM_LAUNCH_CHECK(c);
   m.n_ell = n_ell;
