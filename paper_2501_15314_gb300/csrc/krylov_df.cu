@@ -536,7 +536,7 @@ __global__ void k_round_f32(const double* __restrict__ x, float* __restrict__ v,
 #define IBM_NQ_DISPATCH_DS(nq, KERNEL, ...)                                 \
   do {                                                                      \
     count_launch();                                                         \
-    const int nb_ = red_blocks(m);                                          \
+    const int nb_ = red_blocks(m);   /* (without a sum, k_gemv_ds, too) */   \
     if ((nq) <= 2) KERNEL<2><<<nb_, RT, 0, s>>>(__VA_ARGS__);        \
     else if ((nq) <= 4) KERNEL<4><<<nb_, RT, 0, s>>>(__VA_ARGS__);   \
     else if ((nq) <= 8) KERNEL<8><<<nb_, RT, 0, s>>>(__VA_ARGS__);   \
@@ -548,11 +548,11 @@ __global__ void k_round_f32(const double* __restrict__ x, float* __restrict__ v,
     else KERNEL<kMaxRestart + 1><<<nb_, RT, 0, s>>>(__VA_ARGS__);    \
   } while (0)
 
-// the float4 FP32 kernels, for nq <= 16
-#define IBM_NQ_DISPATCH_SP4(nq, KERNEL, ...)                                       \
+// the float4 FP32 kernels, for nq <= 16, on nb blocks
+#define IBM_NQ_DISPATCH_SP4(nb, nq, KERNEL, ...)                                   \
   do {                                                                             \
     count_launch();                                                                \
-    const dim3 g_(red_blocks(m / 4)), b_(RT);                                      \
+    const dim3 g_(nb), b_(RT);                                                     \
     if ((nq) <= 2) launch_pdl(KERNEL<2>, g_, b_, 0, s, __VA_ARGS__);               \
     else if ((nq) <= 4) launch_pdl(KERNEL<4>, g_, b_, 0, s, __VA_ARGS__);          \
     else if ((nq) <= 8) launch_pdl(KERNEL<8>, g_, b_, 0, s, __VA_ARGS__);          \
@@ -953,7 +953,7 @@ ibm_status fgmres_solve_ds(ibm_ctx* c, const double* b, double* x, const ibm_sol
       const int nb = red_blocks(vec4 && nq <= 16 ? m / 4 : m);
       ph = prof_begin(c, IBM_PROF_MULTIDOT);
       if (vec4 && nq <= 16)
-        IBM_NQ_DISPATCH_SP4(nq, k_multidot_sp4, reinterpret_cast<const float4*>(w1),
+        IBM_NQ_DISPATCH_SP4(nb, nq, k_multidot_sp4, reinterpret_cast<const float4*>(w1),
                             reinterpret_cast<const float4*>(V1), m / 4, nq, m / 4, part);
       else if (single)
         IBM_NQ_DISPATCH_DS(nq, k_multidot_sp, w1, V1, m, nq, m, part);
@@ -966,7 +966,7 @@ ibm_status fgmres_solve_ds(ibm_ctx* c, const double* b, double* x, const ibm_sol
       prof_end(c, ph, (single ? 4.0 : 8.0) * (nq + 1) * (double)m);
       ph = prof_begin(c, IBM_PROF_AXPY_NORM);
       if (vec4 && nq <= 16)
-        IBM_NQ_DISPATCH_SP4(nq, k_axpy_norm_sp4, reinterpret_cast<float4*>(w1),
+        IBM_NQ_DISPATCH_SP4(nb, nq, k_axpy_norm_sp4, reinterpret_cast<float4*>(w1),
                             reinterpret_cast<const float4*>(V1), m / 4, nq, coef_ds, m / 4, part);
       else if (single)
         IBM_NQ_DISPATCH_DS(nq, k_axpy_norm_sp, w1, V1, m, nq, coef_ds, m, part);
@@ -1099,7 +1099,7 @@ ibm_status fgmres_solve_ds(ibm_ctx* c, const double* b, double* x, const ibm_sol
         cy.v[i] = make_float2(yh, (float)(yi - (double)yh));
       }
       if (m % 4 == 0 && jused <= 16 && (reinterpret_cast<uintptr_t>(x) & 15u) == 0)
-        IBM_NQ_DISPATCH_SP4(jused, k_gemv_ds4, reinterpret_cast<double2*>(x),
+        IBM_NQ_DISPATCH_SP4(kRedBlocks, jused, k_gemv_ds4, reinterpret_cast<double2*>(x),
                             reinterpret_cast<const float4*>(Zf), m / 4, jused, cy, m / 4);
       else
         IBM_NQ_DISPATCH_DS(jused, k_gemv_ds, x, Zf, m, jused, cy, m);

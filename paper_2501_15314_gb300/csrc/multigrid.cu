@@ -850,6 +850,127 @@ __global__ void __launch_bounds__(32 * VY) k_prolong_v4(Dims d, Dims dc,
   }
 }
 
+// The prolongation and the first post-smoothing step in one launch, for levels
+// of at most kFuseCells cells: xo = y + w D^{-1} (b - L y), y = x + P xc, four
+// cells and one plane per thread (as k_sweep_v4).  y is formed where it is
+// needed, for the thread's row on three planes and the two rows beside it, from
+// three coarse rows and planes, with the weights 3/4 and 1/4 as 3 a + b per
+// axis and 1/64 in the last step.  These levels wait on latency, and one launch
+// saves more than the repeated interpolation costs: 8.1 us against 4.3 + 5.1 at
+// 64^3, 5.2 against 3.8 + 4.6 at 32^3; at 128^3 it is 21 against 8.2 + 7.0, at
+// 256^3 (in marches of four planes, 128 registers) 108 against 36 + 27.
+constexpr int64_t kFuseCells = 300000;
+
+template <typename TO>
+__global__ void __launch_bounds__(32 * VY) k_prolong_sweep_v4(Dims d, Dims dc,
+                                                              const float* __restrict__ x,
+                                                              const float* __restrict__ xc,
+                                                              const float* __restrict__ b,
+                                                              TO* __restrict__ xo, float w,
+                                                              float h2) {
+  pdl_wait();
+  pdl_trigger();
+  const int lane = threadIdx.x;
+  const int i0 = 4 * (blockIdx.x * 32 + lane);
+  const int j = blockIdx.y * VY + threadIdx.y;
+  const int z = blockIdx.z;
+  const bool act = i0 < d.nx && j < d.ny;
+  const int64_t sy = d.nx, sz = (int64_t)d.nx * d.ny;
+  const int64_t c = (int64_t)z * sz + (int64_t)j * sy + i0;
+  const float4 Z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  // Coarse rows: the parent's, its neighbour on the side the row leans to, and
+  // the one on the other side.  The row lies between the first two (weights 3
+  // and 1); the fine row on the near side has them the other way round, the one
+  // on the far side is the parent with the third.  Likewise the planes.
+  const int J = min(j >> 1, dc.ny - 1), K = z >> 1;
+  const int near = (j & 1) ? 1 : -1, nearz = (z & 1) ? 1 : -1;
+  auto clampi = [](int v, int n) { return min(max(v, 0), n - 1); };
+  const int row[3] = {J * dc.nx, clampi(J + near, dc.ny) * dc.nx, clampi(J - near, dc.ny) * dc.nx};
+  const int csz = dc.nx * dc.ny;
+  const int pl[3] = {K * csz, clampi(K + nearz, dc.nz) * csz, clampi(K - nearz, dc.nz) * csz};
+  const int I0 = i0 >> 1, Im = max(I0 - 1, 0), Ip = min(I0 + 2, dc.nx - 1);
+  const bool hn = act && j + near >= 0 && j + near < d.ny;   // near and far rows exist
+  const bool hf = act && j - near >= 0 && j - near < d.ny;
+  const bool pn = act && z + nearz >= 0 && z + nearz < d.nz;   // near and far planes
+  const bool pf = act && z - nearz >= 0 && z - nearz < d.nz;
+  // all loads first
+  float P[3][3][4];   // [plane][row][column Im, I0, I0 + 1, Ip]
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const float* q = xc + pl[k] + row[r];
+      const bool use = act && (k == 0 || r < 2 || k == 1);   // (the far plane's far row is not)
+      const float2 m = use ? __ldg(reinterpret_cast<const float2*>(q + I0)) : make_float2(0.f, 0.f);
+      P[k][r][0] = use ? __ldg(q + Im) : 0.f;
+      P[k][r][1] = m.x;
+      P[k][r][2] = m.y;
+      P[k][r][3] = use ? __ldg(q + Ip) : 0.f;
+    }
+  const float4 xv0 = act ? ld4(x + c) : Z4;
+  const float4 xa = hn ? ld4(x + c + near * sy) : Z4;
+  const float4 xf = hf ? ld4(x + c - near * sy) : Z4;
+  const float4 xzn = pn ? ld4(x + c + nearz * sz) : Z4;
+  const float4 xzf = pf ? ld4(x + c - nearz * sz) : Z4;
+  const float4 bb = act ? ld4(b + c) : Z4;
+  // x + the four fine values 3 (3 u0 + u1) + (3 v0 + v1) of coarse rows u, v
+  // (weights 3, 1) on planes 0, 1 (weights 3, 1)
+  auto add_row = [](const float (&u0)[4], const float (&u1)[4], const float (&v0)[4],
+                    const float (&v1)[4], float4 xv) {
+    float t[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      t[q] = fmaf(3.f, fmaf(3.f, u0[q], u1[q]), fmaf(3.f, v0[q], v1[q]));
+    constexpr float s = 1.f / 64.f;
+    return make_float4(fmaf(s, fmaf(3.f, t[1], t[0]), xv.x), fmaf(s, fmaf(3.f, t[1], t[2]), xv.y),
+                       fmaf(s, fmaf(3.f, t[2], t[1]), xv.z), fmaf(s, fmaf(3.f, t[2], t[3]), xv.w));
+  };
+  const float4 yc = act ? add_row(P[0][0], P[1][0], P[0][1], P[1][1], xv0) : Z4;
+  const float4 ya = hn ? add_row(P[0][1], P[1][1], P[0][0], P[1][0], xa) : Z4;
+  const float4 yf = hf ? add_row(P[0][0], P[1][0], P[0][2], P[1][2], xf) : Z4;
+  const float4 yzn = pn ? add_row(P[1][0], P[0][0], P[1][1], P[0][1], xzn) : Z4;
+  const float4 yzf = pf ? add_row(P[0][0], P[2][0], P[0][1], P[2][1], xzf) : Z4;
+  float left = __shfl_up_sync(kFull, yc.w, 1);
+  float right = __shfl_down_sync(kFull, yc.x, 1);
+  // across the warp's edge: the neighbour's own value
+  if (lane == 0 || lane == 31) {
+    const int ie = lane == 0 ? i0 - 1 : i0 + 4;
+    float v = 0.f;
+    if (act && ie >= 0 && ie < d.nx) {
+      const int I = ie >> 1, In = clampi((ie & 1) ? I + 1 : I - 1, dc.nx);
+      auto at = [&](int i) {
+        const float* q = xc + pl[0] + i;
+        const float* qn = xc + pl[1] + i;
+        return fmaf(3.f, fmaf(3.f, __ldg(q + row[0]), __ldg(qn + row[0])),
+                    fmaf(3.f, __ldg(q + row[1]), __ldg(qn + row[1])));
+      };
+      v = fmaf(1.f / 64.f, fmaf(3.f, at(I), at(In)), __ldg(x + c + (lane == 0 ? -1 : 4)));
+    }
+    if (lane == 0) left = v;
+    else right = v;
+  }
+  const float xv[4] = {yc.x, yc.y, yc.z, yc.w};
+  const float xl[4] = {left, yc.x, yc.y, yc.z};
+  const float xr[4] = {yc.y, yc.z, yc.w, right};
+  const float va[4] = {ya.x, ya.y, ya.z, ya.w};
+  const float vf[4] = {yf.x, yf.y, yf.z, yf.w};
+  const float vzn[4] = {yzn.x, yzn.y, yzn.z, yzn.w};
+  const float vzf[4] = {yzf.x, yzf.y, yzf.z, yzf.w};
+  const float vb[4] = {bb.x, bb.y, bb.z, bb.w};
+  const int nyz = (j > 0) + (j < d.ny - 1) + (z > 0) + (z < d.nz - 1);
+  float o[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int nn = nyz + (i0 + q > 0) + (i0 + q < d.nx - 1);
+    const float s = (xl[q] + xr[q]) + (va[q] + vf[q]) + (vzn[q] + vzf[q]);
+    o[q] = fmaf(w_over(w, nn), fmaf(h2, vb[q], s - (float)nn * xv[q]), xv[q]);
+  }
+  if (act) st4(xo + c, make_float4(o[0], o[1], o[2], o[3]));
+}
+
+// levels whose prolongation is left to the first post-smoothing step
+bool fuse_ok(const MGLevel& L) { return vec_ok(L.d) && L.m <= kFuseCells; }
+
 // ---------------------------------------------------------------------------
 // The V-cycle below a level of at most kChainCells cells, in one CTA: every
 // level's x, b and a ping-pong buffer live in shared memory, phases are
@@ -1305,15 +1426,23 @@ void pre_smooth(ibm_ctx* c, int l, const TB* b, T* bcopy, T* x, T* t, int p, cud
   }
 }
 
-// one smoothing step src -> dst on level l
+// one smoothing step src -> dst on level l; with xc (where fuse_ok) of
+// src + P xc
 template <typename T, typename TO>
-void sweep_step(ibm_ctx* c, int l, const T* src, const T* b, TO* dst, double w, cudaStream_t s) {
+void sweep_step(ibm_ctx* c, int l, const T* src, const T* xc, const T* b, TO* dst, double w,
+                cudaStream_t s) {
   MGLevel& L = c->lv[l];
   const double h2 = L.h * L.h;
   count_launch();
   if constexpr (std::is_same<T, float>::value) {
     if (vec_ok(L.d)) {
       const int zc = vec_zc(L.d);
+      if (xc) {
+        launch_pdl(k_prolong_sweep_v4<TO>, vec_grid(L.d, 1), dim3(32, VY), 0, s, L.d,
+                   c->lv[l + 1].d, (const float*)src, (const float*)xc, (const float*)b, dst,
+                   (float)w, (float)h2);
+        return;
+      }
       launch_pdl(zc == 4 ? k_sweep_v4<TO, 4> : (zc == 1 ? k_sweep_v4<TO, 1> : k_sweep_v4<TO, 0>),
                  vec_grid(L.d, zc), dim3(32, VY), 0, s, L.d, (const float*)src,
                  (const float*)b, dst, (float)w, (float)h2, zc);
@@ -1325,11 +1454,13 @@ void sweep_step(ibm_ctx* c, int l, const T* src, const T* b, TO* dst, double w, 
              over_count<T>(w), (T)h2, zm);
 }
 
-// Post-smoothing: p Chebyshev steps from x; the last step writes out (which
-// may be FP64 while T is FP32).  Intermediate iterates ping-pong between t and
+// Post-smoothing: p Chebyshev steps from x (from x + P xc where coarse_correct
+// left the prolongation to the first one, xc its result); the last step writes
+// out (which may be FP64 while T is FP32).  Intermediate iterates ping-pong between t and
 // x; out never aliases the step's input.
 template <typename T, typename TO>
-void post_smooth(ibm_ctx* c, int l, const T* b, T* x, T* t, int p, TO* out, cudaStream_t s) {
+void post_smooth(ibm_ctx* c, int l, const T* b, T* x, T* t, int p, TO* out, const T* xc,
+                 cudaStream_t s) {
   MGLevel& L = c->lv[l];
   if (p <= 0) {
     if ((const void*)out != (const void*)x) {
@@ -1345,14 +1476,16 @@ void post_smooth(ibm_ctx* c, int l, const T* b, T* x, T* t, int p, TO* out, cuda
   for (int q = 0; q < p; ++q) {
     const bool last = q == p - 1;
     const int ph = l == 0 ? prof_begin(c, IBM_PROF_MG_SMOOTH_FINE) : -1;
+    const T* pro = q == 0 ? xc : nullptr;
+    const double pro_bytes = pro ? (double)c->lv[l + 1].m * sizeof(T) : 0.0;
     if (last && (const void*)out != (const void*)src) {
-      sweep_step<T, TO>(c, l, src, b, out, w[q], s);
-      prof_end_or_note(c, ph, (double)L.m * (2 * sizeof(T) + sizeof(TO)));
+      sweep_step<T, TO>(c, l, src, pro, b, out, w[q], s);
+      prof_end_or_note(c, ph, (double)L.m * (2 * sizeof(T) + sizeof(TO)) + pro_bytes);
       return;
     }
     T* dst = (src == x) ? t : x;
-    sweep_step<T, T>(c, l, src, b, dst, w[q], s);
-    prof_end_or_note(c, ph, (double)L.m * 3 * sizeof(T));
+    sweep_step<T, T>(c, l, src, pro, b, dst, w[q], s);
+    prof_end_or_note(c, ph, (double)L.m * 3 * sizeof(T) + pro_bytes);
     src = dst;
   }
   // the last step landed in t or x while out aliases the other: copy
@@ -1366,8 +1499,11 @@ void post_smooth(ibm_ctx* c, int l, const T* b, T* x, T* t, int p, TO* out, cuda
 template <typename T>
 void vcycle(ibm_ctx* c, int l, const T* b, T* x, T* t, int pre, int post, cudaStream_t s);
 
+// The coarse-grid correction x += P xc, xc ~ L_c^{-1} R (b - L x).  On small
+// levels with post-smoothing the prolongation is left to its first step
+// (k_prolong_sweep_v4): returns xc then, else null.
 template <typename T>
-void coarse_correct(ibm_ctx* c, int l, const T* b, T* x, int pre, int post, cudaStream_t s) {
+const T* coarse_correct(ibm_ctx* c, int l, const T* b, T* x, int pre, int post, cudaStream_t s) {
   MGLevel& L = c->lv[l];
   MGLevel& C = c->lv[l + 1];
   LevelPtrs<T> cp = ptrs<T>(C);
@@ -1392,6 +1528,7 @@ void coarse_correct(ibm_ctx* c, int l, const T* b, T* x, int pre, int post, cuda
                (T)(1.0 / (L.h * L.h)), zt);
   prof_note(c, (double)L.m * ((xin ? 2 : 1) * sizeof(T)) + (double)C.m * sizeof(T));
   vcycle<T>(c, l + 1, cp.b, cp.x, cp.t, pre, post, s);
+  if (std::is_same<T, float>::value && fuse_ok(L) && pre > 0 && post > 0) return cp.x;
   done = false;
   count_launch();
   if constexpr (std::is_same<T, float>::value) {
@@ -1406,6 +1543,7 @@ void coarse_correct(ibm_ctx* c, int l, const T* b, T* x, int pre, int post, cuda
     launch_pdl(k_prolong<T>, gt, dim3(BX, BY), 0, s, L.d, C.d, (const T*)cp.x, x,
                pre > 0 ? 0 : 1, zt);
   prof_note(c, (double)C.m * sizeof(T) + (double)L.m * ((pre > 0 ? 2 : 1) * sizeof(T)));
+  return nullptr;
 }
 
 constexpr size_t kChainSmemMax = 200 * 1024;
@@ -1507,8 +1645,8 @@ void vcycle(ibm_ctx* c, int l, const T* b, T* x, T* t, int pre, int post, cudaSt
     return;
   }
   if (pre > 0) pre_smooth<T, T>(c, l, b, nullptr, x, t, pre, s);
-  coarse_correct<T>(c, l, b, x, pre, post, s);
-  post_smooth<T, T>(c, l, b, x, t, post, x, s);
+  const T* xc = coarse_correct<T>(c, l, b, x, pre, post, s);
+  post_smooth<T, T>(c, l, b, x, t, post, x, xc, s);
 }
 
 }  // namespace
@@ -1616,12 +1754,12 @@ ibm_status mg_vcycle(ibm_ctx* c, const double* r, double* z, int prec, int pre, 
       k_first<float, double><<<zm_grid(L0.d, zm), dim3(BX, BY), 0, s>>>(L0.d, r, L0.b32, L0.t32,
                                                                         FirstWeights<float>{}, 0, zm);
     }
-    coarse_correct<float>(c, 0, L0.b32, L0.x32, pre, post, s);
-    post_smooth<float, double>(c, 0, L0.b32, L0.x32, L0.t32, post, z, s);
+    const float* xc = coarse_correct<float>(c, 0, L0.b32, L0.x32, pre, post, s);
+    post_smooth<float, double>(c, 0, L0.b32, L0.x32, L0.t32, post, z, xc, s);
   } else {
     if (pre > 0) pre_smooth<double, double>(c, 0, r, nullptr, z, L0.t64, pre, s);
     coarse_correct<double>(c, 0, r, z, pre, post, s);
-    post_smooth<double, double>(c, 0, r, z, L0.t64, post, z, s);
+    post_smooth<double, double>(c, 0, r, z, L0.t64, post, z, (const double*)nullptr, s);
   }
   IBM_LAUNCH_CHECK(c);
   return IBM_OK;
@@ -1646,8 +1784,8 @@ ibm_status mg_vcycle_f32(ibm_ctx* c, const float* r, float* z, int pre, int post
     return IBM_OK;
   }
   if (pre > 0) pre_smooth<float, float>(c, 0, r, nullptr, L0.x32, L0.t32, pre, s);
-  coarse_correct<float>(c, 0, r, L0.x32, pre, post, s);
-  post_smooth<float, float>(c, 0, r, L0.x32, L0.t32, post, z, s);
+  const float* xc = coarse_correct<float>(c, 0, r, L0.x32, pre, post, s);
+  post_smooth<float, float>(c, 0, r, L0.x32, L0.t32, post, z, xc, s);
   IBM_LAUNCH_CHECK(c);
   return IBM_OK;
 }
@@ -1667,8 +1805,8 @@ ibm_status mg_vcycle_pair(ibm_ctx* c, const float2* r, float* z, int pre, int po
     k_first_v4<float2><<<vec_grid(L0.d, zc), dim3(32, VY), 0, s>>>(L0.d, r, L0.b32, L0.t32, 0.f,
                                                                    0.f, 0.f, 0, zc);
   }
-  coarse_correct<float>(c, 0, L0.b32, L0.x32, pre, post, s);
-  post_smooth<float, float>(c, 0, L0.b32, L0.x32, L0.t32, post, z, s);
+  const float* xc = coarse_correct<float>(c, 0, L0.b32, L0.x32, pre, post, s);
+  post_smooth<float, float>(c, 0, L0.b32, L0.x32, L0.t32, post, z, xc, s);
   IBM_LAUNCH_CHECK(c);
   return IBM_OK;
 }

@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(BX * BY) k_grad_axpy(Dims d, FaceGeom g,
 // no-slip ghosts: A e = diag e_c - (nu / h^2) * (sum of neighbours), where the
 // face-normal axis reads the wall faces (which hold 0) and each cell-centred
 // axis adds nu / h^2 to diag for every missing neighbour (ghost = -e_c).
-// Kernels below march along z over ZH planes; blockIdx.z = comp * zchunks +
+// Kernels below march along z over zc planes; blockIdx.z = comp * zchunks +
 // chunk, so one launch covers the three face grids.
 // x[c] for a runtime c in 0..2 without dynamic indexing (which would copy a
 // kernel-parameter struct to local memory)
@@ -350,7 +350,6 @@ __device__ __forceinline__ T sel3(int c, T a, T b, T d) {
   return c == 0 ? a : (c == 1 ? b : d);
 }
 
-constexpr int ZH = 16;
 
 // u_E at (x, y, z) of its own face grid, split into an FP32 pair
 template <int E>
@@ -392,7 +391,7 @@ __device__ __forceinline__ double edge_flux_f64(const FaceGeom& g, const double*
 }
 
 // Right-hand side of the predictor, Eq. (ustar), with the convective term
-// fused in, for the C-faces (one launch per velocity component):
+// fused in, for the C-faces:
 //   rhs = (4 u^n - u^{n-1}) / (2 dt) - G p^n + f - A(u^n) on interior faces
 // (0 on wall faces).  A is the central divergence form on the MAC grid (the
 // cell-centred square of u_C averaged along C, and on the edges the product
@@ -413,22 +412,22 @@ __device__ __forceinline__ double edge_flux_f64(const FaceGeom& g, const double*
 // joins the sum as a pair.  The FP64 result is the exact sum of the pair
 // (one FP64 add).
 // Templating on C makes every stride and boundary test a compile-time case.
+// (The pointers' __restrict__ is the kernels': repeated here it cost 5%.)
 template <int C>
-__global__ void __launch_bounds__(BX * BY) k_predictor_rhs_ds(
-    Dims d, FaceGeom g, const double* __restrict__ un, const double* __restrict__ unm1,
-    const double* __restrict__ pn, const double* __restrict__ fb, int with_adv, dsf c4, dsf c1,
-    dsf cp_h, dsf ca, double* __restrict__ rhs) {
+__device__ __forceinline__ void predictor_rhs(const Dims& d, const FaceGeom& g, const double* un,
+                                              const double* unm1, const double* pn,
+                                              const double* fb, int with_adv, dsf c4, dsf c1,
+                                              dsf cp_h, dsf ca, double* rhs, int z0, int planes) {
   const int lane = threadIdx.x;
   const int i = blockIdx.x * BX + lane;
   const int j = blockIdx.y * BY + threadIdx.y;
   const int n0 = g.n[C][0], n1 = g.n[C][1], n2 = g.n[C][2];
-  const int z0 = blockIdx.z * ZH;
   // u_y and u_z faces share their x-edge fluxes between neighbouring lanes,
   // so lanes past the last face stay in the march (without loads or stores);
   // a row past the last one leaves as a whole warp
   const bool act = i < n0;
   if (j >= n1 || (C == 0 && !act)) return;
-  const int z1 = min(z0 + ZH, n2);
+  const int z1 = min(z0 + planes, n2);
   const int64_t sy = g.sy[C], sz = g.sz[C];
   int64_t f = g.off[C] + (int64_t)z0 * sz + (int64_t)j * sy + i;
   const bool col_wall = (C == 0 && (i == 0 || i == n0 - 1)) || (C == 1 && (j == 0 || j == n1 - 1));
@@ -526,6 +525,39 @@ __global__ void __launch_bounds__(BX * BY) k_predictor_rhs_ds(
     }
     rhs[f] = f2d_exact(v.hi) + f2d_exact(v.lo);
   }
+}
+
+// One component per launch, marches of kRhsPlanes planes.
+constexpr int kRhsPlanes = 16;
+
+template <int C>
+__global__ void __launch_bounds__(BX * BY) k_predictor_rhs_ds(
+    Dims d, FaceGeom g, const double* __restrict__ un, const double* __restrict__ unm1,
+    const double* __restrict__ pn, const double* __restrict__ fb, int with_adv, dsf c4, dsf c1,
+    dsf cp_h, dsf ca, double* __restrict__ rhs) {
+  predictor_rhs<C>(d, g, un, unm1, pn, fb, with_adv, c4, c1, cp_h, ca, rhs,
+                   blockIdx.z * kRhsPlanes, kRhsPlanes);
+}
+
+// The three components in one launch (blockIdx.z = component * zchunks + chunk),
+// for grids that do not fill the chip with marches of 16 planes: one launch per
+// component took 160 us at 32^3 and 243 us at 128^3, where their few blocks left
+// it idle; together, with fewer planes, 9 and 215.
+__global__ void __launch_bounds__(BX * BY) k_predictor_rhs_all(
+    Dims d, FaceGeom g, const double* __restrict__ un, const double* __restrict__ unm1,
+    const double* __restrict__ pn, const double* __restrict__ fb, int with_adv, dsf c4, dsf c1,
+    dsf cp_h, dsf ca, double* __restrict__ rhs, int zc, int zchunks) {
+  const int c = blockIdx.z / zchunks;
+  const int z0 = (blockIdx.z - c * zchunks) * zc;
+  const int n0 = sel3(c, g.n[0][0], g.n[1][0], g.n[2][0]);
+  const int n2 = sel3(c, g.n[0][2], g.n[1][2], g.n[2][2]);
+  if (z0 >= n2 || (int)blockIdx.x * BX >= n0) return;   // block-uniform
+  if (c == 0)
+    predictor_rhs<0>(d, g, un, unm1, pn, fb, with_adv, c4, c1, cp_h, ca, rhs, z0, zc);
+  else if (c == 1)
+    predictor_rhs<1>(d, g, un, unm1, pn, fb, with_adv, c4, c1, cp_h, ca, rhs, z0, zc);
+  else
+    predictor_rhs<2>(d, g, un, unm1, pn, fb, with_adv, c4, c1, cp_h, ca, rhs, z0, zc);
 }
 
 // The predictor's FP32 work arrays hold the faces of a component by colour
@@ -1047,16 +1079,27 @@ void launch_predictor_rhs_adv(Dims d, const double* u_n, const double* u_nm1, co
   const FaceGeom g = make_face_geom(d);
   const dsf c4 = host_ds(4.0 * inv_2dt), c1 = host_ds(inv_2dt), cph = host_ds(inv_h),
             ca = host_ds(0.25 * inv_h);
+  const int64_t bxy = (int64_t)div_up(d.nx + 1, BX) * div_up(d.ny + 1, BY);
+  // planes per thread: about eight blocks per SM (a march forms its first lower
+  // z-flux anew)
+  const int zc = (int)std::min<int64_t>(kRhsPlanes,
+                                        std::max<int64_t>(1, 3 * bxy * (d.nz + 1) / (152 * 8)));
   const dim3 b(BX, BY);
-  count_launch();
-  k_predictor_rhs_ds<0><<<dim3(div_up(d.nx + 1, BX), div_up(d.ny, BY), div_up(d.nz, ZH)), b, 0,
-                          s>>>(d, g, u_n, u_nm1, p_n, f_body, with_adv, c4, c1, cph, ca, rhs);
-  count_launch();
-  k_predictor_rhs_ds<1><<<dim3(div_up(d.nx, BX), div_up(d.ny + 1, BY), div_up(d.nz, ZH)), b, 0,
-                          s>>>(d, g, u_n, u_nm1, p_n, f_body, with_adv, c4, c1, cph, ca, rhs);
-  count_launch();
-  k_predictor_rhs_ds<2><<<dim3(div_up(d.nx, BX), div_up(d.ny, BY), div_up(d.nz + 1, ZH)), b, 0,
-                          s>>>(d, g, u_n, u_nm1, p_n, f_body, with_adv, c4, c1, cph, ca, rhs);
+  if (bxy * (d.nz + 1) < (int64_t)kRhsPlanes * 152 * 8) {   // less than that per component
+    const int zch = div_up(d.nz + 1, zc);
+    count_launch();
+    k_predictor_rhs_all<<<dim3(div_up(d.nx + 1, BX), div_up(d.ny + 1, BY), 3 * zch), b, 0, s>>>(
+        d, g, u_n, u_nm1, p_n, f_body, with_adv, c4, c1, cph, ca, rhs, zc, zch);
+    return;
+  }
+  auto run = [&](auto kernel, int nx, int ny, int nz) {
+    count_launch();
+    kernel<<<dim3(div_up(nx, BX), div_up(ny, BY), div_up(nz, kRhsPlanes)), b, 0, s>>>(
+        d, g, u_n, u_nm1, p_n, f_body, with_adv, c4, c1, cph, ca, rhs);
+  };
+  run(k_predictor_rhs_ds<0>, d.nx + 1, d.ny, d.nz);
+  run(k_predictor_rhs_ds<1>, d.nx, d.ny + 1, d.nz);
+  run(k_predictor_rhs_ds<2>, d.nx, d.ny, d.nz + 1);
 }
 
 }  // namespace ibm
