@@ -1050,13 +1050,14 @@ __device__ ChainSm chain_layout(float* base, const CoarseChain& ch) {
   return S;
 }
 
-// Cells (or 16-byte words) a thread of the chain takes per round: their
-// loads are issued together before their arithmetic or stores, so a round
-// costs about one shared-memory (or L2) latency instead of four.
-constexpr int kChainBatch = 4;
+// 16-byte words a thread of the chain copies per round: their loads are issued
+// together before their stores, so a round costs about one L2 latency instead
+// of four.  (The phases below take one cell at a time: four at a time made the
+// launch 2 us longer.)
+constexpr int kCopyBatch = 4;
 
 // Copies up to four arrays of 16-byte words from global to shared memory as
-// one sequence: each thread loads its kChainBatch words of a round (from
+// one sequence: each thread loads its kCopyBatch words of a round (from
 // whichever array they fall in) before it stores them.
 struct WordSegs {
   uint4* dst[4];
@@ -1066,11 +1067,11 @@ struct WordSegs {
 
 __device__ void copy_segs(const WordSegs& w) {
   const int n = w.end[3];
-  for (int base = threadIdx.x; base < n; base += kChainBatch * (int)blockDim.x) {
-    uint4 v[kChainBatch];
-    int seg[kChainBatch], off[kChainBatch];
+  for (int base = threadIdx.x; base < n; base += kCopyBatch * (int)blockDim.x) {
+    uint4 v[kCopyBatch];
+    int seg[kCopyBatch], off[kCopyBatch];
 #pragma unroll
-    for (int q = 0; q < kChainBatch; ++q) {
+    for (int q = 0; q < kCopyBatch; ++q) {
       const int e = base + q * (int)blockDim.x;
       const int sg = (e >= w.end[0]) + (e >= w.end[1]) + (e >= w.end[2]);
       const int first = sg == 0 ? 0 : (sg == 1 ? w.end[0] : (sg == 2 ? w.end[1] : w.end[2]));
@@ -1080,7 +1081,7 @@ __device__ void copy_segs(const WordSegs& w) {
       if (e < n) v[q] = __ldg(src + off[q]);
     }
 #pragma unroll
-    for (int q = 0; q < kChainBatch; ++q) {
+    for (int q = 0; q < kCopyBatch; ++q) {
       const int e = base + q * (int)blockDim.x;
       const int sg = seg[q];
       uint4* dst = sg == 0 ? w.dst[0] : (sg == 1 ? w.dst[1] : (sg == 2 ? w.dst[2] : w.dst[3]));
@@ -1146,25 +1147,11 @@ __device__ void chain_smooth(const CoarseChain& ch, const ChainSm& S, int l, con
   }
   for (; q < p; ++q) {
     const float wq = w[q];
-    for (int base = threadIdx.x; base < m; base += kChainBatch * nt) {
-      float sn[kChainBatch], xv[kChainBatch], bv[kChainBatch];
-      int nn[kChainBatch];
-#pragma unroll
-      for (int k = 0; k < kChainBatch; ++k) {
-        const int c = base + k * nt;
-        sn[k] = 0.f; xv[k] = 0.f; bv[k] = 0.f; nn[k] = 1;
-        if (c < m) {
-          sn[k] = lap_nb(d, cur, c, nb[c], nn[k]);
-          xv[k] = cur[c];
-          bv[k] = b[c];
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < kChainBatch; ++k) {
-        const int c = base + k * nt;
-        if (c < m)
-          nxt[c] = fmaf(wq * inv_nn(nn[k]), fmaf(h2, bv[k], sn[k] - (float)nn[k] * xv[k]), xv[k]);
-      }
+    for (int c = threadIdx.x; c < m; c += nt) {
+      int nn;
+      const float sn = lap_nb(d, cur, c, nb[c], nn);
+      const float xv = cur[c];
+      nxt[c] = fmaf(wq * inv_nn(nn), fmaf(h2, b[c], sn - (float)nn * xv), xv);
     }
     __syncthreads();
     float* tmp = cur; cur = nxt; nxt = tmp;
@@ -1193,36 +1180,25 @@ __device__ void chain_run(const CoarseChain& ch, const ChainSm& S) {
     // eight threads per coarse cell (one child each), summed by shuffles;
     // the thread count is a multiple of 8, so a coarse cell's eight threads
     // are consecutive lanes of one warp in every round
-    for (int base = 0; base < 8 * mcl; base += kChainBatch * nt) {
-      float r[kChainBatch];
-#pragma unroll
-      for (int k = 0; k < kChainBatch; ++k) {
-        const int tq = base + k * nt + (int)threadIdx.x;
-        r[k] = 0.f;
-        if (tq < 8 * mcl) {
-          const int C = tq >> 3, q = tq & 7;
-          int I, J, K;
-          unpack(pkc[C], I, J, K);
-          const int c =
-              ((2 * K + (q >> 2)) * d.ny + 2 * J + ((q >> 1) & 1)) * d.nx + 2 * I + (q & 1);
-          float v = b[c];
-          if (ch.pre > 0) {
-            int nn;
-            const float sn = lap_nb(d, x, c, nb[c], nn);
-            v -= ((float)nn * x[c] - sn) * ih2;
-          }
-          r[k] = v;
+    for (int base = 0; base < 8 * mcl; base += nt) {
+      const int tq = base + (int)threadIdx.x;
+      float v = 0.f;
+      if (tq < 8 * mcl) {
+        const int C = tq >> 3, q = tq & 7;
+        int I, J, K;
+        unpack(pkc[C], I, J, K);
+        const int c = ((2 * K + (q >> 2)) * d.ny + 2 * J + ((q >> 1) & 1)) * d.nx + 2 * I + (q & 1);
+        v = b[c];
+        if (ch.pre > 0) {
+          int nn;
+          const float sn = lap_nb(d, x, c, nb[c], nn);
+          v -= ((float)nn * x[c] - sn) * ih2;
         }
       }
-#pragma unroll
-      for (int k = 0; k < kChainBatch; ++k) {
-        const int tq = base + k * nt + (int)threadIdx.x;
-        float v = r[k];
-        v += __shfl_xor_sync(0xffffffffu, v, 1);
-        v += __shfl_xor_sync(0xffffffffu, v, 2);
-        v += __shfl_xor_sync(0xffffffffu, v, 4);
-        if (tq < 8 * mcl && (tq & 7) == 0) bc[tq >> 3] = v * 0.125f;
-      }
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      v += __shfl_xor_sync(0xffffffffu, v, 4);
+      if (tq < 8 * mcl && (tq & 7) == 0) bc[tq >> 3] = v * 0.125f;
     }
     __syncthreads();
   }
@@ -1249,34 +1225,20 @@ __device__ void chain_run(const CoarseChain& ch, const ChainSm& S) {
     const uint32_t* pkf = S.pk + ch.off[l];
     const Dims d = ch.d[l], dc = ch.d[l + 1];
     const int m = d.nx * d.ny * d.nz;
-    for (int base = threadIdx.x; base < m; base += kChainBatch * nt) {
-      float v[kChainBatch], xo[kChainBatch];
-#pragma unroll
-      for (int k = 0; k < kChainBatch; ++k) {
-        const int c = base + k * nt;
-        v[k] = 0.f;
-        xo[k] = 0.f;
-        if (c < m) {
-          int i, j, kk;
-          unpack(pkf[c], i, j, kk);
-          const int I = i >> 1, J = j >> 1, K = kk >> 1;
-          const int In = (i & 1) ? min(I + 1, dc.nx - 1) : max(I - 1, 0);
-          const int Jn = (j & 1) ? min(J + 1, dc.ny - 1) : max(J - 1, 0);
-          const int Kn = (kk & 1) ? min(K + 1, dc.nz - 1) : max(K - 1, 0);
-          auto X = [&](int a, int bb, int cc) { return xc[(cc * dc.ny + bb) * dc.nx + a]; };
-          const float a00 = 0.75f * X(I, J, K) + 0.25f * X(In, J, K);
-          const float a01 = 0.75f * X(I, Jn, K) + 0.25f * X(In, Jn, K);
-          const float a10 = 0.75f * X(I, J, Kn) + 0.25f * X(In, J, Kn);
-          const float a11 = 0.75f * X(I, Jn, Kn) + 0.25f * X(In, Jn, Kn);
-          v[k] = 0.75f * (0.75f * a00 + 0.25f * a01) + 0.25f * (0.75f * a10 + 0.25f * a11);
-          if (ch.pre > 0) xo[k] = x[c];
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < kChainBatch; ++k) {
-        const int c = base + k * nt;
-        if (c < m) x[c] = ch.pre > 0 ? xo[k] + v[k] : v[k];
-      }
+    for (int c = threadIdx.x; c < m; c += nt) {
+      int i, j, kk;
+      unpack(pkf[c], i, j, kk);
+      const int I = i >> 1, J = j >> 1, K = kk >> 1;
+      const int In = (i & 1) ? min(I + 1, dc.nx - 1) : max(I - 1, 0);
+      const int Jn = (j & 1) ? min(J + 1, dc.ny - 1) : max(J - 1, 0);
+      const int Kn = (kk & 1) ? min(K + 1, dc.nz - 1) : max(K - 1, 0);
+      auto X = [&](int a, int bb, int cc) { return xc[(cc * dc.ny + bb) * dc.nx + a]; };
+      const float a00 = 0.75f * X(I, J, K) + 0.25f * X(In, J, K);
+      const float a01 = 0.75f * X(I, Jn, K) + 0.25f * X(In, Jn, K);
+      const float a10 = 0.75f * X(I, J, Kn) + 0.25f * X(In, J, Kn);
+      const float a11 = 0.75f * X(I, Jn, Kn) + 0.25f * X(In, Jn, Kn);
+      const float v = 0.75f * (0.75f * a00 + 0.25f * a01) + 0.25f * (0.75f * a10 + 0.25f * a11);
+      x[c] = ch.pre > 0 ? x[c] + v : v;
     }
     __syncthreads();
     chain_smooth(ch, S, l, ch.wpost, ch.post, false);
