@@ -14,13 +14,15 @@ import torch
 from . import _lib
 from ._lib import IBM_PREC_FP32, IBM_PREC_FP64, check
 
+_CUDA = torch.device("cuda")   # the current device
+
 __all__ = ["IBMSolver", "RigidSpheres", "IBM_PREC_FP32", "IBM_PREC_FP64"]
 
 
 def _ptr(t: torch.Tensor, dtype=torch.float64, numel=None, name="tensor") -> int:
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
-    if t.device.type != "cuda" or t.dtype != dtype or not t.is_contiguous():
+    if not t.is_cuda or t.dtype != dtype or not t.is_contiguous():
         raise ValueError(f"{name} must be a contiguous CUDA {dtype} tensor")
     if numel is not None and t.numel() != numel:
         raise ValueError(f"{name} has {t.numel()} elements, expected {numel}")
@@ -92,6 +94,9 @@ class IBMSolver:
         h = 1.0 / nx if h is None else h
         self.nx, self.ny, self.nz, self.h, self.Re, self.dt = nx, ny, nz, h, Re, dt
         self.stream = stream if stream is not None else torch.cuda.current_stream()
+        # its handle and device, to tell the caller's current stream from it
+        # without making a Stream object in every call (2 us of a call's 20)
+        self._on = (self.stream.cuda_stream, self.stream.device_index)
         g = _lib.ibm_grid_desc(nx, ny, nz, h, Re, dt)
         ctx = C.c_void_p()
         st = self.lib.ibm_create(C.byref(g), C.c_void_p(self.stream.cuda_stream), C.byref(ctx))
@@ -101,6 +106,7 @@ class IBMSolver:
         self.m = self.lib.ibm_num_cells(ctx)
         self.nf = self.lib.ibm_num_faces(ctx)
         self.n_markers = 0
+        self._refused = False   # the last marker set or two-way step failed
 
     # -- lifetime ---------------------------------------------------------
     def close(self):
@@ -119,26 +125,34 @@ class IBMSolver:
         stream is another one, the call is ordered after it (where the inputs
         and the freshly allocated outputs were written) and the current
         stream after the call (where the results are read)."""
+        dev = torch.cuda.current_device()
+        if (torch._C._cuda_getCurrentRawStream(dev), dev) == self._on:
+            return getattr(self.lib, name)(self.ctx, *args)
         cur = torch.cuda.current_stream()
-        other = cur != self.stream
-        if other:
-            self.stream.wait_stream(cur)
+        self.stream.wait_stream(cur)
         status = getattr(self.lib, name)(self.ctx, *args)
-        if other:
-            cur.wait_stream(self.stream)
+        cur.wait_stream(self.stream)
         return status
 
-    def _cells(self, **kw):
-        return torch.empty(self.m, dtype=torch.float64, device="cuda", **kw)
+    def _cells(self):
+        return torch.empty(self.m, dtype=torch.float64, device=_CUDA)
 
     def _faces(self):
-        return torch.empty(self.nf, dtype=torch.float64, device="cuda")
+        return torch.empty(self.nf, dtype=torch.float64, device=_CUDA)
+
+    def _markers(self):
+        """A marker vector for an entry point that writes all of it (nothing of
+        it where the library refused the last set)."""
+        make = torch.zeros if self._refused else torch.empty
+        return make(3 * self.n_markers, dtype=torch.float64, device=_CUDA)
 
     # -- setup ------------------------------------------------------------
     def set_markers(self, X: torch.Tensor):
         X = X.reshape(3, -1) if X.numel() else X
         n = X.shape[1] if X.numel() else 0
+        self._refused = True
         check(self._call("ibm_set_markers", n, _ptr(X, name="X") if n else None), self.ctx)
+        self._refused = False
         self.n_markers = n
         self._X = X
 
@@ -184,8 +198,7 @@ class IBMSolver:
         return out
 
     def interp(self, u, out=None):
-        out = torch.zeros(3 * self.n_markers, dtype=torch.float64, device="cuda") \
-            if out is None else out
+        out = self._markers() if out is None else out
         if self.n_markers:
             check(self._call("ibm_interp", _ptr(u, numel=self.nf, name="u"),
                                       _ptr(out, name="U")), self.ctx)
@@ -210,8 +223,7 @@ class IBMSolver:
         return out
 
     def force_correction(self, p, rhs_F, out=None):
-        out = torch.zeros(3 * self.n_markers, dtype=torch.float64, device="cuda") \
-            if out is None else out
+        out = self._markers() if out is None else out
         if self.n_markers:
             check(self._call("ibm_force_correction", _ptr(p, numel=self.m, name="p"),
                                                 _ptr(rhs_F, name="rhs_F"),
@@ -283,6 +295,7 @@ class IBMSolver:
         fo.xi, fo.tol, fo.max_inner = float(xi), float(tol), int(max_inner)
         fo.criterion = int(criterion)
         st = _lib.ibm_fsi_stats()
+        self._refused = True
         status = self._call("ibm_fsi_step",
             spheres.n, spheres.arr, n, _ptr(L0, numel=nmk, name="L0"),
             _ptr(body_id, dtype=torch.int32, numel=n, name="body_id"),
@@ -294,6 +307,7 @@ class IBMSolver:
             C.byref(o), C.byref(fo), C.byref(st))
         if raise_on_error:
             check(status, self.ctx)
+        self._refused = False
         self.n_markers = n
         return out, dict(inner=st.inner, fgmres_iters=st.fgmres_iters, ratio=st.ratio,
                          helm_iters=st.helm_iters, helm_relres=st.helm_relres, status=status)
