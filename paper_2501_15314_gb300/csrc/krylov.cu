@@ -10,6 +10,7 @@
 // Reductions are two-stage with a grid set by the length (red_blocks blocks,
 // fixed-order tree inside each block, then one fixed-order tree per output):
 // results are bitwise reproducible run to run.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -431,18 +432,22 @@ ibm_status fgmres_solve(ibm_ctx* c, const double* b, double* x, const ibm_solve_
     g[0] = beta;
     int jused = 0;
     bool breakdown = false;
-    for (int j = 0; j < restart && total < o->maxit; ++j) {
+    // Iteration j's kernels; the Hessenberg column goes to the host mirror (its
+    // dot products in one of two buffers by the parity of j) and an event marks
+    // the iteration's end.
+    auto launch_iter = [&](int j) -> ibm_status {
       double* vj = V + (int64_t)j * m;
       double* zj = Z + (int64_t)j * m;
       double* w = V + (int64_t)(j + 1) * m;
+      ibm_status sv;
       const double mk0 = prof_mark(c);
       int ph = prof_begin(c, IBM_PROF_VCYCLE);
-      if ((stt = mg_vcycle(c, vj, zj, o->precond_prec, o->mg_pre, o->mg_post)) != IBM_OK)
-        return stt;
+      if ((sv = mg_vcycle(c, vj, zj, o->precond_prec, o->mg_pre, o->mg_post)) != IBM_OK) return sv;
       prof_end_span(c, ph, mk0);
-      if ((stt = schur_apply(c, zj, w)) != IBM_OK) return stt;
+      if ((sv = schur_apply(c, zj, w)) != IBM_OK) return sv;
       ph = prof_begin(c, IBM_PROF_MULTIDOT);
-      launch_multidot(w, V, m, j + 1, m, part, raw, s, nrm2, coef, hmirror(c, hr));
+      launch_multidot(w, V, m, j + 1, m, part, raw, s, nrm2, coef,
+                      hmirror(c, hr + (2 + (j & 1)) * kOutStride));
       prof_end(c, ph, 8.0 * (j + 2) * (double)m);
       ph = prof_begin(c, IBM_PROF_AXPY_NORM);
       launch_axpy_norm(w, V, m, j + 1, coef, m, part, nrm2 + j + 1, s,
@@ -450,14 +455,43 @@ ibm_status fgmres_solve(ibm_ctx* c, const double* b, double* x, const ibm_solve_
       prof_end(c, ph, 8.0 * (j + 3) * (double)m);
       if (o->reorth) {
         launch_multidot(w, V, m, j + 1, m, part, raw2, s, nrm2, coef2,
-                        hmirror(c, hr + 2 * kOutStride));
+                        hmirror(c, hr + (5 + (j & 1)) * kOutStride));
         launch_axpy_norm(w, V, m, j + 1, coef2, m, part, nrm2 + j + 1, s,
                          hmirror(c, hr + 4 * kOutStride + j + 1));
       }
       IBM_LAUNCH_CHECK(c);
-      IBM_CUDA(c, cudaStreamSynchronize(s));
-      for (int i = 0; i <= j; ++i)
-        Hm(i, j) = (hr[i] + (o->reorth ? hr[2 * kOutStride + i] : 0.0)) / rn[i];
+      IBM_CUDA(c, cudaEventRecord(c->ev_iter[j & 1], s));
+      return IBM_OK;
+    };
+    // As in the single-precision cycles (krylov_df.cu), iteration j + 1, which
+    // needs nothing from the host, is launched before iteration j's column is
+    // read while the residual estimate, shrinking at the fastest rate seen so
+    // far, cannot reach the threshold at iteration j: the device does not idle
+    // during the host's read, Givens update and launches (FP64 step at 32^3:
+    // 1.46 ms instead of 1.57; adjoint at 128^3: 15.4 instead of 16.0; at 256^3
+    // the iteration is long enough to hide them, 28.7 and 28.8).  A wrong guess
+    // costs the unused iteration; the iterates and their number do not depend on
+    // the guesses.  The exact and sign-consistent forms wait on the host in
+    // every product.
+    const double thresh = o->rtol * bnorm;
+    const bool ahead = c->cmode == IBM_CMODE_SCALAR;
+    double prev = beta, rate = 0.05;   // assumed until a ratio has been seen
+    bool have_rate = false, next_launched = false;
+    if (restart > 0 && total < o->maxit) {
+      if ((stt = launch_iter(0)) != IBM_OK) return stt;
+      next_launched = true;
+    }
+    for (int j = 0; next_launched; ++j) {
+      const bool can_next = j + 1 < restart && total + 1 < o->maxit;
+      next_launched = false;
+      if (ahead && can_next && prev * rate > 4.0 * thresh) {
+        if ((stt = launch_iter(j + 1)) != IBM_OK) return stt;
+        next_launched = true;
+      }
+      IBM_CUDA(c, cudaEventSynchronize(c->ev_iter[j & 1]));
+      const double* hraw = hr + (2 + (j & 1)) * kOutStride;
+      const double* hraw2 = hr + (5 + (j & 1)) * kOutStride;
+      for (int i = 0; i <= j; ++i) Hm(i, j) = (hraw[i] + (o->reorth ? hraw2[i] : 0.0)) / rn[i];
       const double hn = std::sqrt(hr[4 * kOutStride + j + 1]);
       if (!std::isfinite(hn)) return set_err(c, IBM_ERR_NAN, "non-finite Arnoldi vector");
       Hm(j + 1, j) = hn;
@@ -477,8 +511,18 @@ ibm_status fgmres_solve(ibm_ctx* c, const double* b, double* x, const ibm_solve_
       g[j] = cs[j] * g[j];
       ++total;
       jused = j + 1;
-      if (st && total - 1 < IBM_HIST_MAX) st->relres_hist[total - 1] = std::fabs(g[j + 1]) / bnorm;
-      if (std::fabs(g[j + 1]) / bnorm <= o->rtol || hn == 0.0) break;
+      const double res = std::fabs(g[j + 1]);
+      if (st && total - 1 < IBM_HIST_MAX) st->relres_hist[total - 1] = res / bnorm;
+      if (res / bnorm <= o->rtol || hn == 0.0) break;
+      if (prev > 0.0) {
+        rate = have_rate ? std::min(rate, res / prev) : res / prev;
+        have_rate = true;
+      }
+      prev = res;
+      if (!next_launched && can_next) {
+        if ((stt = launch_iter(j + 1)) != IBM_OK) return stt;
+        next_launched = true;
+      }
     }
     if (jused > 0) {
       for (int i = jused - 1; i >= 0; --i) {
