@@ -52,14 +52,15 @@ UNIT = "solves/s"
 # null).  Below 1: part of a launch's output is still in the 129 MB L2 when
 # it ends (written back later, often never: the next kernel reads it there).
 NCU_TRAFFIC_RATIO = {
-    # predictor FP32 Chebyshev step (mode 1): 631.7 + 181.4 MB for 808.5 MB
-    "helm_sweep": 1.0058,
+    # predictor FP32 half-step, two launches: 302.9 + 72.9 and 302.9 + 70.4 MB
+    # for 404.2 MB each
+    "helm_sweep": 0.9265,
     # finest-level smoothing, one V-cycle: k_first_v4 67.2 + 27.1 MB and the
     # two k_sweep_v4 134.2 + 38.8 and 134.2 + 37.4 MB, for 134.2 + 2 x 201.3 MB
     "mg_smooth_fine": 0.8177,
     # FP32 Gram-Schmidt at basis lengths 6 and 7
-    "multidot": 1.0042,
-    "axpy_norm": 0.9744,
+    "multidot": 1.0120,
+    "axpy_norm": 0.9733,
     # Schur Laplacian class per step: 14 k_lap_ds (69.4 + 24.2 MB for 134.2 MB)
     # and 2 k_laplacian_fx forming b - L x (268.5 + 108.4 MB for 402.7 MB)
     "laplacian_f64": 0.7691,
@@ -107,8 +108,8 @@ def measured_peaks():
 # the Schur solve (the metric's unit); the roofline record names the one of
 # them that takes the most time.
 ROOFLINE_CLASSES = {
-    "k_helm_cheb_v4 (predictor FP32 Chebyshev step: read e, e_old, r; write e_new)":
-        "helm_sweep",
+    ("k_helm_half (predictor FP32 red-black Chebyshev half-step: the other colour of e, "
+     "r and e of this colour read; e of this colour written)"): "helm_sweep",
     "k_multidot_sp4 (Gram-Schmidt multi-dot on FP32 vectors, float4: w and V_0..V_j)":
         "multidot",
     "k_axpy_norm_sp4 (Gram-Schmidt axpy+norm on FP32 vectors, float4: V_0..V_j, w in/out)":

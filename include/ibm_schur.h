@@ -96,7 +96,7 @@ typedef enum { IBM_ARNOLDI_FP64 = 0, IBM_ARNOLDI_DS = 1, IBM_ARNOLDI_FP32 = 2 } 
  * IBM_CMODE_EXACT: S = L + B^T C^{-1} B, b = RHS_p + B^T C^{-1} RHS_F,
  *   F' = C^{-1}(B p' - RHS_F) (Eqs. (SchurPrimal)-(SchurPrimalF)), the
  *   operator of the spectral theorem of Sec. 5; C^{-1} by conjugate
- *   gradients on C (matrix-free R^T R) to c_rtol inside every product.
+ *   gradients on C = R^T R to c_rtol inside every product.
  * IBM_CMODE_CONSISTENT: the sign-consistent system [[L, -B^T], [B, -C]]
  *   that the update of Eq. (u_n_plus_1) implies when G^T u^{n+1} = 0 and
  *   R^T u^{n+1} = U^Gamma are imposed exactly: S = L - B^T C^{-1} B,
@@ -251,17 +251,20 @@ ibm_status ibm_apply_schur_opts(ibm_ctx* ctx, const double* v, double* out,
                                 const ibm_solve_opts* opts, int64_t* c_iters);
 
 /* s = C^{-1} t with C = R^T R ([3][n_markers] device vectors, t and s must
- * not alias): conjugate gradients on C, products matrix-free (spread to the
- * shell faces, interpolate back), to ||t - C s|| <= c_rtol ||t|| within
+ * not alias): conjugate gradients on C, to ||t - C s|| <= c_rtol ||t|| within
  * c_maxit iterations (IBM_ERR_NOT_CONVERGED otherwise, s holds the last
- * iterate).  iters may be NULL.  Synchronises. */
+ * iterate).  The first call after ibm_set_markers forms C's rows (about 36
+ * entries per marker and component at spacing h); many or dense markers
+ * are multiplied matrix-free (spread to the shell faces, interpolate back).
+ * iters may be NULL.  Synchronises. */
 ibm_status ibm_apply_c_inverse(ibm_ctx* ctx, const double* t, double* s, double c_rtol,
                                int32_t c_maxit, int32_t* iters);
 
 /* One one-way SIMPLE-IBM time step (Sec. 3.1) with the markers last set:
  *   1. predictor (Eq. (ustar)): (3/(2dt) - Lap/Re) u* = (4u^n - u^{n-1})/(2dt)
- *      - G p^n + R F^n - (u.grad u)^n + f_body, solved by FP64 defect
- *      correction around FP32 Chebyshev sweeps to helm_rtol;
+ *      - G p^n + R F^n - (u.grad u)^n + f_body, solved by defect correction
+ *      (double-single residual) around FP32 red-black Chebyshev half-steps
+ *      to helm_rtol;
  *   2. RHS_p = (3/(2dt)) G^T u*, RHS_F = (3/(2dt)) (R^T u* - U_gamma);
  *   3. ibm_solve_schur on b = RHS_p + 2 B^T RHS_F (scalar C mode;
  *      RHS_p +- B^T C^{-1} RHS_F in the EXACT / CONSISTENT modes);
@@ -480,8 +483,8 @@ enum {
   IBM_PROF_STEP = 7,           /* whole ibm_step                            */
   IBM_PROF_MARKER_BUILD = 8,   /* ibm_set_markers                           */
   IBM_PROF_MG_SMOOTH_FINE = 9, /* one finest-level smoothing sweep kernel   */
-  IBM_PROF_HELM_SWEEP = 10,    /* one inner FP32 Chebyshev step of the
-                                  predictor (middle steps only)             */
+  IBM_PROF_HELM_SWEEP = 10,    /* one inner FP32 Chebyshev half-step (one
+                                  colour) of the predictor                  */
   IBM_PROF_ADJOINT = 11,       /* whole ibm_adjoint_step                    */
   IBM_PROF_FSI = 12,           /* whole ibm_fsi_step                        */
   IBM_PROF_NCLASS = 16

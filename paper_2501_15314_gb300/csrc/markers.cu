@@ -187,7 +187,7 @@ __global__ void k_fill(Dims d, MkView mk, const int32_t* __restrict__ start, int
   key[pos] = (int32_t)(k * 64 + s);
 }
 
-// Sorts each shell cell's segment (one warp per segment): the keys are
+// Sorts each shell cell's segment (a warp per two segments): the keys are
 // distinct, so a key's place is the number of smaller keys in the segment;
 // segments of up to 64 keys are ranked in registers (two keys per lane),
 // longer ones by an insertion sort in lane 0.  Makes the entry order
