@@ -528,6 +528,18 @@ __device__ __forceinline__ float ell_combine_f32(float v) {
   return v;
 }
 
+// Orders of traversal.  A kernel that runs over arrays larger than L2 (129 MB)
+// from the other end than the kernel before it finds what that one touched last
+// still in L2; in the same order it finds nothing.  past_l2: the bytes that two
+// such kernels share do not fit beside what they write (where they do, the
+// order does not matter).  Measured, a step: 256^3 15.87 -> 15.50 ms, 384^3
+// 42.54 -> 42.07.
+inline int past_l2(int64_t bytes) { return bytes > 96 * (int64_t)1000000; }
+// the block's z index, counted from the end of the grid if rev
+__device__ __forceinline__ int z_block(int rev) {
+  return rev ? (int)(gridDim.z - 1 - blockIdx.z) : (int)blockIdx.z;
+}
+
 // Programmatic dependent launch: a kernel launched with launch_pdl may be
 // scheduled while its predecessor in the stream is still finishing, and
 // pdl_wait() (first statement of such a kernel) blocks until that

@@ -484,14 +484,14 @@ template <typename TO, int ZC = 0>
 __global__ void __launch_bounds__(32 * VY) k_sweep_v4(Dims d, const float* __restrict__ x,
                                                       const float* __restrict__ b,
                                                       TO* __restrict__ xo, float w, float h2,
-                                                      int zc) {
+                                                      int zc, int rev) {
   pdl_wait();
   pdl_trigger();
   const int lane = threadIdx.x;
   const int i0 = 4 * (blockIdx.x * 32 + lane);
   const int j = blockIdx.y * VY + threadIdx.y;
   const bool act = i0 < d.nx && j < d.ny;
-  const int z0 = blockIdx.z * zc;
+  const int z0 = z_block(rev) * zc;
   const int z1 = min(z0 + zc, d.nz);
   const int64_t sy = d.nx, sz = (int64_t)d.nx * d.ny;
   int64_t c = (int64_t)z0 * sz + (int64_t)j * sy + i0;
@@ -734,14 +734,14 @@ __global__ void __launch_bounds__(32 * VY, 4) k_restrict_v4(Dims d, Dims dc,
                                                          const float* __restrict__ x,
                                                          const float* __restrict__ b,
                                                          float* __restrict__ bcoarse, float inv_h2,
-                                                         int zcc) {
+                                                         int zcc, int rev) {
   pdl_wait();
   pdl_trigger();
   const int lane = threadIdx.x;
   const int i0 = 4 * (blockIdx.x * 32 + lane);
   const int J = blockIdx.y * VY + threadIdx.y;
   const bool act = i0 < d.nx && J < dc.ny;
-  const int K0 = blockIdx.z * zcc;
+  const int K0 = z_block(rev) * zcc;
   const int K1 = min(K0 + zcc, dc.nz);
   const int64_t sy = d.nx, sz = (int64_t)d.nx * d.ny;
   const float4 Z4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1375,7 +1375,8 @@ void pre_smooth(ibm_ctx* c, int l, const TB* b, T* bcopy, T* x, T* t, int p, cud
         launch_pdl(zc == 4 ? k_sweep_v4<float, 4>
                            : (zc == 1 ? k_sweep_v4<float, 1> : k_sweep_v4<float, 0>),
                    vec_grid(L.d, zc), dim3(32, VY), 0, s, L.d,
-                   (const float*)cur, (const float*)bb, nxt, (float)w[q], (float)h2, zc);
+                   (const float*)cur, (const float*)bb, nxt, (float)w[q], (float)h2, zc,
+                   (p - 1 - q) & past_l2(8 * L.m));
     }
     if (!vec)
       launch_pdl(k_sweep<T, T, T>, zm_grid(L.d, zm), dim3(BX, BY), 0, s, L.d, (const T*)cur, bb,
@@ -1392,7 +1393,7 @@ void pre_smooth(ibm_ctx* c, int l, const TB* b, T* bcopy, T* x, T* t, int p, cud
 // src + P xc
 template <typename T, typename TO>
 void sweep_step(ibm_ctx* c, int l, const T* src, const T* xc, const T* b, TO* dst, double w,
-                cudaStream_t s) {
+                int rev, cudaStream_t s) {
   MGLevel& L = c->lv[l];
   const double h2 = L.h * L.h;
   count_launch();
@@ -1407,7 +1408,7 @@ void sweep_step(ibm_ctx* c, int l, const T* src, const T* xc, const T* b, TO* ds
       }
       launch_pdl(zc == 4 ? k_sweep_v4<TO, 4> : (zc == 1 ? k_sweep_v4<TO, 1> : k_sweep_v4<TO, 0>),
                  vec_grid(L.d, zc), dim3(32, VY), 0, s, L.d, (const float*)src,
-                 (const float*)b, dst, (float)w, (float)h2, zc);
+                 (const float*)b, dst, (float)w, (float)h2, zc, rev & past_l2(8 * L.m));
       return;
     }
   }
@@ -1441,12 +1442,12 @@ void post_smooth(ibm_ctx* c, int l, const T* b, T* x, T* t, int p, TO* out, cons
     const T* pro = q == 0 ? xc : nullptr;
     const double pro_bytes = pro ? (double)c->lv[l + 1].m * sizeof(T) : 0.0;
     if (last && (const void*)out != (const void*)src) {
-      sweep_step<T, TO>(c, l, src, pro, b, out, w[q], s);
+      sweep_step<T, TO>(c, l, src, pro, b, out, w[q], !(q & 1), s);
       prof_end_or_note(c, ph, (double)L.m * (2 * sizeof(T) + sizeof(TO)) + pro_bytes);
       return;
     }
     T* dst = (src == x) ? t : x;
-    sweep_step<T, T>(c, l, src, pro, b, dst, w[q], s);
+    sweep_step<T, T>(c, l, src, pro, b, dst, w[q], !(q & 1), s);
     prof_end_or_note(c, ph, (double)L.m * 3 * sizeof(T) + pro_bytes);
     src = dst;
   }
@@ -1478,7 +1479,7 @@ const T* coarse_correct(ibm_ctx* c, int l, const T* b, T* x, int pre, int post, 
       launch_pdl(k_restrict_v4,
                  dim3(div_up(L.d.nx / 4, 32), div_up(C.d.ny, VY), div_up(C.d.nz, zcc)),
                  dim3(32, VY), 0, s, L.d, C.d, (const float*)xin, (const float*)b, cp.b,
-                 (float)(1.0 / (L.h * L.h)), zcc);
+                 (float)(1.0 / (L.h * L.h)), zcc, past_l2(8 * L.m));
       done = true;
     }
   }

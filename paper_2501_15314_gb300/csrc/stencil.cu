@@ -625,12 +625,14 @@ template <int LX, bool FULL>
 __global__ void __launch_bounds__(kHelmThreads) k_helm_half(HelmGeom p, int zc, int zchunks,
                                                             int col, float* e,
                                                             const float* __restrict__ r, float nu,
-                                                            float4 w, float omw, int old_zero) {
+                                                            float4 w, float omw, int old_zero,
+                                                            int rev) {
   pdl_wait();
   pdl_trigger();
   constexpr int kRows = kHelmThreads / LX;
-  const int c = blockIdx.z / zchunks;
-  const int z0 = (blockIdx.z - c * zchunks) * zc;
+  const int bz = z_block(rev);
+  const int c = bz / zchunks;
+  const int z0 = (bz - c * zchunks) * zc;
   const int n1 = sel3(c, p.n[0][1], p.n[1][1], p.n[2][1]);
   const int n2 = sel3(c, p.n[0][2], p.n[1][2], p.n[2][2]);
   if (z0 >= n2 || (int)blockIdx.y * kRows >= n1) return;   // block-uniform
@@ -1048,7 +1050,7 @@ void launch_helm_half(Dims d, int col, float* e, const float* r, double a, doubl
   const auto k8 = full ? k_helm_half<8, true> : k_helm_half<8, false>;
   launch_pdl(h.lx == 32 ? k32 : (h.lx == 16 ? k16 : k8), h.grid, h.block, 0, s, make_helm_geom(d),
              h.zc, h.zch, col, e, r, (float)nu_h2, helm_weights(a, nu_h2, omega),
-             (float)(1.0 - omega), old_zero ? 1 : 0);
+             (float)(1.0 - omega), old_zero ? 1 : 0, col & past_l2(24 * (int64_t)d.nx * d.ny * d.nz));
 }
 
 int64_t launch_helm_resid(Dims d, const float* e, float* rhi, float* rlo, double a, double nu_h2,
