@@ -186,6 +186,12 @@ const char* ibm_last_error(const ibm_ctx* ctx);
 int64_t ibm_num_cells(const ibm_ctx* ctx);
 int64_t ibm_num_faces(const ibm_ctx* ctx);
 
+/* n = number of markers that the context holds, the length of a component of
+ * its marker vectors: those of the last ibm_set_markers or ibm_fsi_step that
+ * came to set its markers, 0 where they were refused.  Host only; the last
+ * error's message stays. */
+ibm_status ibm_num_markers(const ibm_ctx* ctx, int64_t* n);
+
 /* Sets the Lagrangian markers (Sec. 2.3): X is device [3][n_markers] FP64
  * positions.  Builds the per-marker Roma weights of Eq. (delta) for the three
  * velocity components and a cell-sorted marker list used by the deterministic

@@ -99,6 +99,7 @@ SIGNATURES = [
     ("ibm_last_error", C.c_char_p, [_P]),
     ("ibm_num_cells", C.c_int64, [_P]),
     ("ibm_num_faces", C.c_int64, [_P]),
+    ("ibm_num_markers", C.c_int, [_P, C.POINTER(C.c_int64)]),
     ("ibm_set_markers", C.c_int, [_P, C.c_int64, _P]),
     ("ibm_apply_laplacian", C.c_int, [_P, _P, _P]),
     ("ibm_apply_schur", C.c_int, [_P, _P, _P]),

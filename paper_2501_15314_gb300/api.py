@@ -106,7 +106,7 @@ class IBMSolver:
         self.m = self.lib.ibm_num_cells(ctx)
         self.nf = self.lib.ibm_num_faces(ctx)
         self.n_markers = 0
-        self._refused = False   # the last marker set or two-way step failed
+        self._refused = False   # the library holds no markers: it refused the last set
 
     # -- lifetime ---------------------------------------------------------
     def close(self):
@@ -140,6 +140,18 @@ class IBMSolver:
     def _faces(self):
         return torch.empty(self.nf, dtype=torch.float64, device=_CUDA)
 
+    def _after_markers(self, ok, n):
+        """Takes over the marker count that the library holds after a call that
+        sets n markers: a refused set leaves none, a call refused before it
+        the earlier ones, and one that fails after it its own.  Marker vectors
+        are sized by the count; where the set was refused the library writes
+        none of them, and ``n_markers`` is left to the caller."""
+        held = C.c_int64()
+        self.lib.ibm_num_markers(self.ctx, C.byref(held))
+        self._refused = held.value == 0 and not (ok and n == 0)
+        if not self._refused:
+            self.n_markers = held.value
+
     def _markers(self):
         """A marker vector for an entry point that writes all of it (nothing of
         it where the library refused the last set)."""
@@ -150,10 +162,9 @@ class IBMSolver:
     def set_markers(self, X: torch.Tensor):
         X = X.reshape(3, -1) if X.numel() else X
         n = X.shape[1] if X.numel() else 0
-        self._refused = True
-        check(self._call("ibm_set_markers", n, _ptr(X, name="X") if n else None), self.ctx)
-        self._refused = False
-        self.n_markers = n
+        status = self._call("ibm_set_markers", n, _ptr(X, name="X") if n else None)
+        self._after_markers(status == _lib.IBM_OK, n)
+        check(status, self.ctx)
         self._X = X
 
     # -- operators --------------------------------------------------------
@@ -295,7 +306,6 @@ class IBMSolver:
         fo.xi, fo.tol, fo.max_inner = float(xi), float(tol), int(max_inner)
         fo.criterion = int(criterion)
         st = _lib.ibm_fsi_stats()
-        self._refused = True
         status = self._call("ibm_fsi_step",
             spheres.n, spheres.arr, n, _ptr(L0, numel=nmk, name="L0"),
             _ptr(body_id, dtype=torch.int32, numel=n, name="body_id"),
@@ -305,10 +315,11 @@ class IBMSolver:
             _ptr(out["X"], numel=nmk, name="X"), _ptr(out["u"], numel=self.nf, name="u"),
             _ptr(out["p"], numel=self.m, name="p"), _ptr(out["F"], numel=nmk, name="F"),
             C.byref(o), C.byref(fo), C.byref(st))
+        self._after_markers(status == _lib.IBM_OK, n)
         if raise_on_error:
             check(status, self.ctx)
-        self._refused = False
-        self.n_markers = n
+        if self._refused:
+            self.n_markers = n
         return out, dict(inner=st.inner, fgmres_iters=st.fgmres_iters, ratio=st.ratio,
                          helm_iters=st.helm_iters, helm_relres=st.helm_relres, status=status)
 

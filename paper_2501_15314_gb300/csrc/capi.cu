@@ -458,6 +458,11 @@ const char* ibm_last_error(const ibm_ctx* c) { return c ? c->err.c_str() : "null
 
 int64_t ibm_num_cells(const ibm_ctx* c) { return c ? c->m : 0; }
 int64_t ibm_num_faces(const ibm_ctx* c) { return c ? c->nf : 0; }
+ibm_status ibm_num_markers(const ibm_ctx* c, int64_t* n) {
+  if (!c || !n) return IBM_ERR_ARG;
+  *n = c->mk.n;
+  return IBM_OK;
+}
 
 ibm_status ibm_set_markers(ibm_ctx* c, int64_t n, const double* X) {
   if (check_ctx(c) != IBM_OK) return IBM_ERR_ARG;
