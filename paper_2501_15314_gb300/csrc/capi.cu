@@ -430,8 +430,8 @@ ibm_status ibm_create(const ibm_grid_desc* g, void* stream, ibm_ctx** out) {
     delete c;
     return IBM_ERR_NOMEM;
   }
-  // the predictor's FP32 arrays: a row's padding is never written and must
-  // read as 0
+  // the predictor's FP32 arrays: a row's padding must read as 0 (the solves
+  // write nothing else to it)
   for (float* buf : {c->hr, c->hl, c->he[0], c->he[1]})
     if (cudaMemset(buf, 0, sizeof(float) * helm_fp32_size(c->d)) != cudaSuccess) ok = false;
   ibm_status st = ok ? mg_setup(c) : IBM_ERR_CUDA;

@@ -567,7 +567,8 @@ __global__ void __launch_bounds__(BX * BY) k_predictor_rhs_all(
 // x-neighbours of element q of one colour are the elements q and q - 1 (i
 // even) or q and q + 1 (i odd) of the other colour's row, the y- and
 // z-neighbours its elements q of the rows beside.  Padding, and the wall face
-// i = nx of u_x when nx is odd, hold 0; when nx is even that face has no place.
+// i = nx of u_x when nx is odd, hold 0 (also where faces hold infinities or
+// NaN); when nx is even that face has no place.
 struct HelmGeom {
   int nx;
   int nq;              // elements per row and colour, ceil(nx / 2)
@@ -617,8 +618,8 @@ __device__ __forceinline__ int ghosts(bool centred, int x, int n) {
 // (Golub and Varga's cyclic Chebyshev semi-iterative method).
 // Four elements per thread (float4), LX threads per row, z-neighbours from the
 // march, x by one shuffle, y through L1.  old_zero: e of this colour is zero
-// and not read.  Weights are 0 at wall faces and past a row's end, where e is
-// and stays 0.  FULL: nx is a multiple of 8, so only the first and last element
+// and not read.  Weights are 0 at wall faces, where e is and stays 0.  FULL: nx is
+// a multiple of 8, so rows have no padding and only the first and last element
 // of a row can differ from the row's others.  Bound by HBM and instruction
 // issue: 16 B per updated face, 8 B per face of the grid.
 template <int LX, bool FULL>
@@ -703,6 +704,14 @@ __global__ void __launch_bounds__(kHelmThreads) k_helm_half(HelmGeom p, int zc, 
                omw * old.z);
     o.w = fmaf(wt[3], fmaf(nu, (oc.w + (s ? side : oc.z)) + (ym.w + yp.w) + (om.w + on.w), rr.w),
                omw * old.w);
+    if (!FULL) {
+      // The row's padding stays 0 whatever its neighbours hold (a zero weight
+      // times an infinity would not): later solves read it and never write it.
+      if ((dead >> sp) & 1) o.x = 0.f;
+      if ((dead >> (sp + 1)) & 1) o.y = 0.f;
+      if ((dead >> (sp + 2)) & 1) o.z = 0.f;
+      if ((dead >> (sp + 3)) & 1) o.w = 0.f;
+    }
     if (act) *reinterpret_cast<float4*>(ec) = o;
     om = oc;
     oc = on;

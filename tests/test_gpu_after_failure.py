@@ -8,6 +8,42 @@ from gpu_cases import dev, host
 
 pytestmark = pytest.mark.gpu
 
+
+@pytest.mark.parametrize("grid", [(12, 8, 8), (16, 8, 8), (20, 12, 8), (18, 14, 10), (9, 7, 8)],
+                         ids=lambda g: "x".join(map(str, g)))
+def test_step_after_an_overflowing_one(cuda_device, grid):
+    """The right-hand side 4 u^n / (2 dt) = 4e31 is finite in FP64 and past the
+    range of its FP32 parts (2^101), so the predictor ends with IBM_ERR_NAN;
+    a valid step after it gives the bits of one on a fresh solver."""
+    from paper_2501_15314_gb300 import _lib
+    from paper_2501_15314_gb300.api import IBMSolver
+    nx, ny, nz = grid
+    rng = np.random.default_rng(nx)
+    none = dev(np.zeros(1))
+
+    def solver():
+        return IBMSolver(nx, ny, nz, 1.0 / nx, Re=50.0, dt=5e-4)
+
+    def step(s, u, **kw):
+        return s.step(u, zero, cells, none, none, f, raise_on_error=False, with_advection=0, **kw)
+
+    a, b = solver(), solver()
+    zero, cells = dev(np.zeros(a.nf)), dev(np.zeros(a.m))
+    f = dev(rng.standard_normal(a.nf))
+    good = dev(rng.standard_normal(a.nf))
+    ref, st = step(a, good)
+    assert st["status"] == _lib.IBM_OK
+    for _ in range(2):
+        _, st = step(b, dev(np.full(a.nf, 1e28)))
+        assert st["status"] == _lib.IBM_ERR_NAN
+        out, st = step(b, good)
+        assert st["status"] == _lib.IBM_OK
+        for k in ("u", "p"):
+            np.testing.assert_array_equal(host(out[k]), host(ref[k]))
+    a.close()
+    b.close()
+
+
 N = 24
 
 
