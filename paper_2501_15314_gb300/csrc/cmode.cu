@@ -463,30 +463,32 @@ ibm_status form_rows(ibm_ctx* c, CgArgs& a, int sms, bool& rows) {
     launch_to_host(mk.c_off + mk.n, c->host_flag_dev, sizeof(int32_t), str);
     IBM_LAUNCH_CHECK(c);
     IBM_CUDA(c, cudaStreamSynchronize(str));
-    mk.c_n = c->host_flag[0];
-    mk.c_formed = true;
-    if (mk.c_n > (int64_t)kRowMax * mk.n) mk.c_n = 0;   // too long: the spread form
-    if (mk.c_n > mk.c_val_cap) {
+    int64_t entries = c->host_flag[0];
+    mk.c_n = 0;
+    if (entries > (int64_t)kRowMax * mk.n) entries = 0;   // too long: the spread form
+    if (entries > mk.c_val_cap) {
       cudaFree(mk.c_val);
       mk.c_val_cap = 0;
       // the values, then the columns
-      if (cudaMalloc(&mk.c_val, (3 * sizeof(double) + sizeof(int32_t)) * mk.c_n) != cudaSuccess) {
+      if (cudaMalloc(&mk.c_val, (3 * sizeof(double) + sizeof(int32_t)) * entries) != cudaSuccess) {
         cudaGetLastError();
         mk.c_val = nullptr;
-        mk.c_n = 0;   // no room for the rows: the spread form
+        entries = 0;   // no room for the rows: the spread form
       } else {
-        mk.c_val_cap = mk.c_n;
+        mk.c_val_cap = entries;
       }
     }
-    mk.c_col = reinterpret_cast<int32_t*>(mk.c_val + 3 * mk.c_n);
-    if (mk.c_n > 0) {
-      a.n_val = mk.c_n;
+    if (entries > 0) {
+      mk.c_col = reinterpret_cast<int32_t*>(mk.c_val + 3 * entries);
+      a.n_val = entries;
       count_launch();
       k_c_rows<true><<<blocks, TPB, 0, str>>>(c->d, mk.n, mk.n_entries, mk.org, c->cell_start,
                                               mk.entry_key, a, nullptr, mk.c_off, mk.c_col,
                                               mk.c_val);
       IBM_LAUNCH_CHECK(c);
     }
+    mk.c_n = entries;      // rows that were not filled are never taken as formed
+    mk.c_formed = true;
   }
   rows = mk.c_n > 0;
   a.off = mk.c_off;
