@@ -1026,8 +1026,8 @@ ibm_status markers_build(ibm_ctx* c, int64_t n, const double* X) {
                                                      m.cw32, reinterpret_cast<SlotWeights*>(m.slot),
                                                      c->dev_flag);
   IBM_LAUNCH_CHECK(c);
-  m.n = n;
-  const MkView mv = view(m);
+  MkView mv = view(m);
+  mv.n = n;   // the context holds them once their lists are complete
   // counting sort of (marker, slot) pairs by cell: counts, then one
   // reduction and one scan-and-list pass over the counts for the segment
   // starts and the shell-cell list, then the fill (which takes the counts
@@ -1053,11 +1053,9 @@ ibm_status markers_build(ibm_ctx* c, int64_t n, const double* X) {
   launch_to_host(c->dev_flag, c->host_flag_dev + 2, sizeof(int32_t), s);
   IBM_LAUNCH_CHECK(c);
   IBM_CUDA(c, cudaStreamSynchronize(s));
-  if (c->host_flag[2] != 0) {
-    m.n = 0;
+  if (c->host_flag[2] != 0)
     return set_err(c, IBM_ERR_MARKER_DOMAIN,
                    "a marker's delta support touches a wall face or leaves the grid");
-  }
   const int64_t ne = c->host_flag[0], ns = c->host_flag[1];
   st = grow_entries(c, ne);
   if (st != IBM_OK) return st;
@@ -1092,6 +1090,7 @@ ibm_status markers_build(ibm_ctx* c, int64_t n, const double* X) {
                                              m.ell_len, perm, n_ell, m.ell_key,
                                              m.ell_coef, m.ell_coef32, m.ell_sw, m.ell_any);
   IBM_LAUNCH_CHECK(c);
+  m.n = n;
   m.n_ell = n_ell;
   m.n_entries = ne;
   m.n_shell = ns;
