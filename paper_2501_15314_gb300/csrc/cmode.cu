@@ -70,10 +70,12 @@ struct CgArgs {
 
 // Grid-wide barrier with the sum of v over the grid's threads, in a fixed order
 // (each warp, the block's warps, the blocks).  The blocks' arrivals are counted
-// up to round * blocks; the partial sums alternate between two arrays, as a
-// block may enter the next barrier while others still read this one's.  Every
-// block is resident (cooperative launch), so the barrier ends; should it not, a
-// limit on the polls sets the error flag and all blocks leave.
+// up to round * blocks, modulo 2^32 (14 million iterations of 152 blocks): the
+// counts compared differ by less than two rounds, so the sign of their
+// difference tells which is ahead.  The partial sums alternate between two
+// arrays, as a block may enter the next barrier while others still read this
+// one's.  Every block is resident (cooperative launch), so the barrier ends;
+// should it not, a limit on the polls sets the error flag and all blocks leave.
 // One warp forms the total and, from it and num, the scalar the caller needs:
 // total / num (OVER), num / total (else), 0 where the divisor is.  An FP64
 // operation has 64 cycles of latency and takes a warp 16 cycles of its SM's
@@ -109,9 +111,9 @@ __device__ bool grid_sum(const CgArgs& a, double v, double num, unsigned& round,
       int polls = 0;
       do {
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.bar) : "memory");
-      } while (seen < want && ++polls < kSpinLimit);
-      ok = seen >= want;
-      if (seen < want) atomicExch(a.bar + 1, 1u);
+      } while ((int)(seen - want) < 0 && ++polls < kSpinLimit);
+      ok = (int)(seen - want) >= 0;
+      if (!ok) atomicExch(a.bar + 1, 1u);
     }
     __syncwarp();
     t = 0.0;
