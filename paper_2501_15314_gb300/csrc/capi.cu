@@ -415,14 +415,11 @@ ibm_status ibm_create(const ibm_grid_desc* g, void* stream, ibm_ctx** out) {
             cudaMalloc(&c->gstate, sizeof(double) * GState::kSize) == cudaSuccess &&
             cudaHostAlloc(&c->host_gstate, sizeof(double) * GState::kSize, cudaHostAllocMapped) ==
                 cudaSuccess &&
-            cudaHostGetDevicePointer(&c->host_gstate_dev, c->host_gstate, 0) == cudaSuccess;
-  {
-    // partial sums of the fused predictor residual norm (one per block)
-    const int64_t nb = (int64_t)div_up(g->nx + 1, 32) * div_up(g->ny + 1, 8) * 3 *
-                       div_up(g->nz + 1, 16);
-    c->helm_part_n = nb * (kMaxRestart + 2);
-    ok = ok && cudaMalloc(&c->helm_part, sizeof(double) * c->helm_part_n) == cudaSuccess;
-  }
+            cudaHostGetDevicePointer(&c->host_gstate_dev, c->host_gstate, 0) == cudaSuccess &&
+            // one partial sum per block of either norm's kernel
+            cudaMalloc(&c->helm_part,
+                       sizeof(double) * std::max(helm_resid_blocks(c->d),
+                                                 gradt_norm2_blocks(c->d))) == cudaSuccess;
   c->cell_touch = c->scan_tmp + nscan;
   if (!ok) {
     cudaGetLastError();
@@ -669,13 +666,8 @@ static ibm_status step_impl(ibm_ctx* c, const double* u_n, const double* u_nm1, 
   // 6. diagnostics: both squared norms go to the host mirror, one round trip
   double* dslot = c->red_out + 7 * (kMaxRestart + 2);
   // ||G^T u||^2 from per-block sums of squares (G^T u itself is not stored)
-  if (gradt_norm2_blocks(c->d) <= c->helm_part_n) {
-    const int64_t nb = launch_gradt_norm2(c->d, u_np1, inv_h, c->helm_part, str);
-    launch_final_reduce(c->helm_part, (int)nb, dslot, str, c->host_red_dev, 1);
-  } else {
-    launch_gradient_t(c->d, u_np1, c->c1, inv_h, str);
-    launch_dot(c->c1, c->c1, c->m, c->red_part, dslot, str, c->host_red_dev);
-  }
+  const int64_t nb = launch_gradt_norm2(c->d, u_np1, inv_h, c->helm_part, str);
+  launch_final_reduce(c->helm_part, (int)nb, dslot, str, c->host_red_dev, 1);
   if (n > 0) {
     launch_interp(c, u_np1, mk.t2);
     count_launch();

@@ -166,8 +166,8 @@ struct ibm_ctx {
   double* defer_mean = nullptr;
   double* host_red = nullptr;      // mapped pinned mirror of red_out (host address)
   double* host_red_dev = nullptr;  // its device address
-  double* helm_part = nullptr;     // per-block partials of the predictor norm
-  int64_t helm_part_n = 0;         // its length (also holds the divergence norm's partials)
+  double* helm_part = nullptr;     // per-block partials of the predictor's residual norm
+                                   // and of the divergence norm
 
   // Krylov bases
   double* V = nullptr;             // [(kMaxRestart + 1)][m]
@@ -282,7 +282,9 @@ void launch_helm_start(Dims d, const double* r64, float scale, double a, double 
 void launch_helm_half(Dims d, int col, float* e, const float* r, double a, double nu_h2,
                       double omega, bool old_zero, cudaStream_t s);
 // (rhi, rlo) -= A e in double-single, per-block sums of the new hi^2 in part
-// (returns their number), D^{-1} of the new residual on colour 0 into en
+// (returns their number, helm_resid_blocks(d)), D^{-1} of the new residual on
+// colour 0 into en
+int64_t helm_resid_blocks(Dims d);
 int64_t launch_helm_resid(Dims d, const float* e, float* rhi, float* rlo, double a, double nu_h2,
                           float* en, double* part, cudaStream_t s);
 // u = 2^k (e + pe) (pe may be null), 0 on the walls; add: u += 2^k e

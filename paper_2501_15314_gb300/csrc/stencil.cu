@@ -1062,14 +1062,22 @@ void launch_helm_half(Dims d, int col, float* e, const float* r, double a, doubl
              (float)(1.0 - omega), old_zero ? 1 : 0, col & past_l2(24 * (int64_t)d.nx * d.ny * d.nz));
 }
 
+// two elements of each colour per thread
+static HelmShape helm_resid_shape(Dims d) { return helm_shape(d, div_up(d.nx, 4)); }
+
+int64_t helm_resid_blocks(Dims d) {
+  const HelmShape h = helm_resid_shape(d);
+  return (int64_t)h.grid.x * h.grid.y * h.grid.z;
+}
+
 int64_t launch_helm_resid(Dims d, const float* e, float* rhi, float* rlo, double a, double nu_h2,
                           float* en, double* part, cudaStream_t s) {
-  const HelmShape h = helm_shape(d, div_up(d.nx, 4));
+  const HelmShape h = helm_resid_shape(d);
   const auto k = h.lx == 32 ? k_helm_resid<32> : (h.lx == 16 ? k_helm_resid<16> : k_helm_resid<8>);
   count_launch();
   k<<<h.grid, h.block, 0, s>>>(make_helm_geom(d), h.zc, h.zch, e, rhi, rlo, host_ds(a),
                                host_ds(nu_h2), helm_weights(a, nu_h2, 1.0), en, part);
-  return (int64_t)h.grid.x * h.grid.y * h.grid.z;
+  return helm_resid_blocks(d);
 }
 
 void launch_helm_flush(Dims d, const float* e, const float* pe, int k, bool add, double* u,
