@@ -16,6 +16,11 @@ from ._lib import IBM_PREC_FP32, IBM_PREC_FP64, check
 
 _CUDA = torch.device("cuda")   # the current device
 
+# handle of a device's current stream: torch's own accessor, or, where a version
+# has none by that name, through a Stream object (2 us more per call)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream",
+                      lambda dev: torch.cuda.current_stream(dev).cuda_stream)
+
 __all__ = ["IBMSolver", "RigidSpheres", "IBM_PREC_FP32", "IBM_PREC_FP64"]
 
 
@@ -126,7 +131,7 @@ class IBMSolver:
         and the freshly allocated outputs were written) and the current
         stream after the call (where the results are read)."""
         dev = torch.cuda.current_device()
-        if (torch._C._cuda_getCurrentRawStream(dev), dev) == self._on:
+        if (_raw_stream(dev), dev) == self._on:
             return getattr(self.lib, name)(self.ctx, *args)
         cur = torch.cuda.current_stream()
         self.stream.wait_stream(cur)
