@@ -9,10 +9,10 @@
 // (about 5e2 at Lagrangian spacing h, 2e5 at h / 1.38 for a sphere of radius
 // 0.3 on 32^3), which is why the paper uses C^{-1} ~ 2 I in production.
 //
-// A solve takes hundreds of iterations of a microsecond's work each, so a whole
+// A solve takes hundreds of iterations of microseconds' work each, so a whole
 // solve is one cooperative launch of at most one block per SM whose phases are
 // separated by grid-wide barriers, which carry the partial sums of the two dot
-// products with them.  Two forms:
+// products with them.  Three forms:
 //   rows: C's rows are formed once per marker set (the overlaps of the markers'
 //     supports, about 36 per marker at spacing h) and kept until the markers
 //     change; an iteration is one product and two barriers.  The vectors'
@@ -22,10 +22,16 @@
 //     markers than the grid's registers hold, or rows longer than kRowMax on
 //     average (markers much denser than h), where the rows cost more memory
 //     and time than the spread's 64 + 27 weights.
+//   launched: the spread form's phases as kernels of full grids, nine per
+//     iteration, the residual read by the host every four.  For more than
+//     kOneLaunchMax markers, where an iteration waits on memory for longer than
+//     nine launches take and one block per SM keeps too few loads in flight.
 // Measured on GB300, us per iteration: rows 11.5 at 1158 markers, 14 at 4632,
-// 24 at 12000, the two barriers with their sums taking about 8 of them; spread
-// 56 at 26100; launched kernel by kernel (ten per iteration, the residual read
-// by the host every four) 50 at 1158.
+// 24 at 12000, 41 at 25900 (launched 50, 61 at 6000, 73 at 25900), the two
+// barriers with their sums taking about 8 of them.  Spread, on spheres at
+// spacing h, with blocks of 512 threads / of 1024 / launched: 57 / 47 / 78 at
+// 26100 markers, 139 / 104 / 122 at 60000, 310 / 217 / 217 at 150000, 653 / 445 /
+// 401 at 330000; 10^6 markers in a volume 1630 / 1252 / 989.
 #include "ibm_internal.cuh"
 
 #include <algorithm>
@@ -39,6 +45,8 @@ namespace {
 constexpr int TPB = 256;
 constexpr int kCgThreads = 512;
 constexpr int kCgWarps = kCgThreads / 32;
+constexpr int kCgWide = 1024;  // threads of the spread form's larger blocks
+constexpr int64_t kOneLaunchMax = 150000;   // markers of the one-launch forms
 constexpr int kCheck = 4;      // the residual is tested every four iterations
 constexpr int kRowLanes = 4;   // lanes per row and component
 constexpr int kRowUnits = 32 / kRowLanes;   // rows a warp takes at once
@@ -88,7 +96,7 @@ struct GridSum {
 
 template <bool OVER>
 __device__ bool grid_sum(const CgArgs& a, double v, double num, unsigned& round, GridSum& out) {
-  __shared__ double sh[kCgWarps];
+  __shared__ double sh[kCgWide / 32];
   __shared__ GridSum all;
   __shared__ int ok;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
@@ -385,8 +393,12 @@ __device__ __forceinline__ double cg_interp(const CgArgs& a, int dc, int64_t k) 
 }
 
 // s = C^{-1} t through the faces.  A thread owns the same marker values in
-// every phase; the spread alone reads others'.
-__global__ void __launch_bounds__(kCgThreads, 1) k_cg_spread(const CgArgs a) {
+// every phase; the spread alone reads others'.  Blocks of 512 threads where
+// these are enough for a warp per group of shell cells (128 registers: more loads
+// in flight per warp; 600 markers at spacing h / 4 42 us an iteration, against
+// 47 with 64 registers), of 1024 where there is more work than that.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) k_cg_spread(const CgArgs a) {
   const int64_t n3 = 3 * a.n;
   const int64_t first =
       ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
@@ -441,6 +453,77 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg_spread(const CgArgs a) {
     a.out[1] = rr;
     a.out[2] = (double)it;
   }
+}
+
+// ---- launched ----
+
+__global__ void __launch_bounds__(TPB) k_spread_set(const CgArgs a) { cg_spread(a); }
+
+__global__ void k_cg_alpha(const double* __restrict__ rr, const double* __restrict__ pq,
+                           double* __restrict__ alpha) {
+  alpha[0] = pq[0] != 0.0 ? rr[0] / pq[0] : 0.0;
+}
+
+// s += alpha p, r -= alpha q
+__global__ void __launch_bounds__(TPB) k_cg_update(const CgArgs a,
+                                                   const double* __restrict__ alpha) {
+  const double f = alpha[0];
+  for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < 3 * a.n;
+       i += (int64_t)gridDim.x * TPB) {
+    a.s[i] = fma(f, a.p[i], a.s[i]);
+    a.r[i] = fma(-f, a.q[i], a.r[i]);
+  }
+}
+
+// p = r + (rr_new / rr) p
+__global__ void __launch_bounds__(TPB) k_cg_direction(const CgArgs a,
+                                                      const double* __restrict__ rr,
+                                                      const double* __restrict__ rr_new) {
+  const double beta = rr[0] > 0.0 ? rr_new[0] / rr[0] : 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < 3 * a.n;
+       i += (int64_t)gridDim.x * TPB)
+    a.p[i] = fma(beta, a.p[i], a.r[i]);
+}
+
+// The solve kernel by kernel; sc: four device scalars (<r, r> before and after
+// the iteration in turn, <p, q>, alpha).  tt = <t, t>, rr = the last <r, r> read.
+ibm_status cg_launched(ibm_ctx* c, const CgArgs& a, double* sc, double& tt, double& rr, int& it) {
+  cudaStream_t str = c->stream;
+  const int64_t n = 3 * a.n;
+  const int grid = (int)std::min<int64_t>(div_up(n, TPB), kRedBlocks);
+  launch_zero(a.s, sizeof(double) * n, str);
+  launch_copy(a.r, a.t, sizeof(double) * n, str);
+  launch_copy(a.p, a.t, sizeof(double) * n, str);
+  launch_dot(a.t, a.t, n, c->red_part, sc, str, c->host_red_dev);
+  IBM_LAUNCH_CHECK(c);
+  IBM_CUDA(c, cudaStreamSynchronize(str));
+  tt = rr = c->host_red[0];
+  if (!std::isfinite(tt) || tt == 0.0) return IBM_OK;
+  while (it < a.maxit) {
+    double* now = sc + (it & 1);
+    double* next = sc + 1 - (it & 1);
+    count_launch();
+    k_spread_set<<<div_up(32 * ell_groups(a.n_shell), TPB), TPB, 0, str>>>(a);
+    launch_interp(c, a.face, a.q);
+    launch_dot(a.p, a.q, n, c->red_part, sc + 2, str);
+    count_launch();
+    k_cg_alpha<<<1, 1, 0, str>>>(now, sc + 2, sc + 3);
+    count_launch();
+    k_cg_update<<<grid, TPB, 0, str>>>(a, sc + 3);
+    ++it;
+    const bool test = it % kCheck == 0 || it == a.maxit;
+    launch_dot(a.r, a.r, n, c->red_part, next, str, test ? c->host_red_dev : nullptr);
+    if (test) {
+      IBM_LAUNCH_CHECK(c);
+      IBM_CUDA(c, cudaStreamSynchronize(str));
+      rr = c->host_red[0];
+      if (!(rr > a.rtol2 * tt)) break;   // small, or not a number
+    }
+    count_launch();
+    k_cg_direction<<<grid, TPB, 0, str>>>(a, now, next);
+  }
+  IBM_LAUNCH_CHECK(c);
+  return IBM_OK;
 }
 
 // C's rows for the markers set (a.off, a.col, a.val), formed at the first
@@ -510,7 +593,7 @@ ibm_status c_solve(ibm_ctx* c, const double* t, double* s, double rtol, int maxi
   if (iters_out) *iters_out = 0;
   if (n == 0) return IBM_OK;
   if (!c->cg_bar) {
-    if (cudaMalloc(&c->cg_bar, 2 * sizeof(unsigned)) != cudaSuccess) {
+    if (cudaMalloc(&c->cg_bar, 2 * sizeof(unsigned) + 4 * sizeof(double)) != cudaSuccess) {
       cudaGetLastError();
       c->cg_bar = nullptr;
       return set_err(c, IBM_ERR_NOMEM, "CG barrier allocation failed");
@@ -549,23 +632,36 @@ ibm_status c_solve(ibm_ctx* c, const double* t, double* s, double rtol, int maxi
   bool rows;
   const ibm_status st = form_rows(c, a, sms, rows);
   if (st != IBM_OK) return st;
-  // at most one block per SM (all resident), and no more warps than the
-  // markers give work: an idle warp still takes part in the barriers
-  const int64_t warps = rows ? div_up(n, kRowUnits)
-                             : std::max<int64_t>(ell_groups(mk.n_shell), div_up(n, 32));
-  const int blocks = (int)std::min<int64_t>(warps, sms);
-  const int threads = 32 * (int)std::min<int64_t>(kCgWarps, div_up(warps, blocks));
-  launch_zero(c->cg_bar, 2 * sizeof(unsigned), str);
-  count_launch();
-  void* args[] = {&a};
-  IBM_CUDA(c, cudaLaunchCooperativeKernel(rows ? (const void*)k_cg_rows : (const void*)k_cg_spread,
-                                          dim3(blocks), dim3(threads), args, 0, str));
-  launch_to_host(a.bar + 1, c->host_flag_dev, sizeof(unsigned), str);
-  IBM_LAUNCH_CHECK(c);
-  IBM_CUDA(c, cudaStreamSynchronize(str));
-  if (c->host_flag[0]) return set_err(c, IBM_ERR_CUDA, "grid barrier of the CG on C timed out");
-  const double tt = c->host_red[0], rr = c->host_red[1];
-  const int it = (int)c->host_red[2];
+  double tt = 0.0, rr = 0.0;
+  int it = 0;
+  if (!rows && mk.n > kOneLaunchMax) {
+    const ibm_status sl =
+        cg_launched(c, a, reinterpret_cast<double*>(c->cg_bar + 2), tt, rr, it);
+    if (sl != IBM_OK) return sl;
+  } else {
+    // at most one block per SM (all resident), and no more warps than the
+    // markers give work: an idle warp still takes part in the barriers
+    const int64_t warps = rows ? div_up(n, kRowUnits)
+                               : std::max<int64_t>(ell_groups(mk.n_shell), div_up(n, 32));
+    const int blocks = (int)std::min<int64_t>(warps, sms);
+    const int64_t each = div_up(warps, blocks);
+    const bool wide = !rows && each > kCgWarps;
+    const int threads = 32 * (int)std::min<int64_t>(wide ? kCgWide / 32 : kCgWarps, each);
+    const void* kernel = rows ? (const void*)k_cg_rows
+                              : (wide ? (const void*)k_cg_spread<kCgWide>
+                                      : (const void*)k_cg_spread<kCgThreads>);
+    launch_zero(c->cg_bar, 2 * sizeof(unsigned), str);
+    count_launch();
+    void* args[] = {&a};
+    IBM_CUDA(c, cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(threads), args, 0, str));
+    launch_to_host(a.bar + 1, c->host_flag_dev, sizeof(unsigned), str);
+    IBM_LAUNCH_CHECK(c);
+    IBM_CUDA(c, cudaStreamSynchronize(str));
+    if (c->host_flag[0]) return set_err(c, IBM_ERR_CUDA, "grid barrier of the CG on C timed out");
+    tt = c->host_red[0];
+    rr = c->host_red[1];
+    it = (int)c->host_red[2];
+  }
   if (!std::isfinite(tt)) return set_err(c, IBM_ERR_NAN, "non-finite right-hand side of C s = t");
   if (tt == 0.0) return IBM_OK;
   if (!std::isfinite(rr)) return set_err(c, IBM_ERR_NAN, "non-finite CG residual on C");

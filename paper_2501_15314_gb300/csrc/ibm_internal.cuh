@@ -193,7 +193,7 @@ struct ibm_ctx {
   double c_rtol = 1e-14;
   int c_maxit = 500;
   int64_t c_iters = 0;             // inner CG iterations since the call began
-  unsigned* cg_bar = nullptr;      // [2] grid barrier of the CG on C
+  unsigned* cg_bar = nullptr;      // CG on C: [2] grid barrier, then 4 FP64 scalars
 
   // event timing of kernel classes (ibm_profile_enable)
   bool prof_on = false;

@@ -1,9 +1,11 @@
 """C^{-1} = (R^T R)^{-1} where its conjugate gradients take one form or the
 other: the last marker count of the rows form and the first of the spread form
-(a lane group holds at most four rows), a count that fills its third and fourth
-rows, cells with more than the 32 entries a warp reads at once, the two sets
-too dense for rows (by the cells' entries, and by the rows' own length), and
-rows formed again when the markers change.
+(a lane group holds at most four rows; 8192 and 8193, which other tests have,
+are no limit of it), the last of the one-launch forms and the first solved kernel
+by kernel, counts that fill the third and fourth rows, cells with more than the
+32 entries a warp reads at once, the two sets too dense for rows (by the cells'
+entries, and by the rows' own length), and rows formed again when the markers
+change.
 
 C s is recomputed with the library's own spread and interpolation.  Bounds: at
 marker spacing h as for the sizes below the limit, 2.2e-16 ||s|| sqrt(500)
@@ -27,12 +29,13 @@ def _limit():
     return torch.cuda.get_device_properties(0).multi_processor_count * 16 * 8 * 4 // 3
 
 
-@pytest.mark.parametrize("which", ["rounds3", "rounds4", "last_rows", "first_spread"])
+@pytest.mark.parametrize("which", ["rounds3", "rounds4", "last_rows", "first_spread",
+                                   "last_one_launch", "first_launched"])
 def test_large_counts(cuda_device, which):
     from paper_2501_15314_gb300.api import IBMSolver
     count = {"rounds3": _limit() * 5 // 8, "rounds4": _limit() * 7 // 8, "last_rows": _limit(),
-             "first_spread": _limit() + 1}[which]
-    n = 128
+             "first_spread": _limit() + 1, "last_one_launch": 150000, "first_launched": 150001}[which]
+    n = 128 if count < 100000 else 256
     s = IBMSolver(n)
     s.set_markers(dev(wl.fibonacci_sphere(count, float(np.sqrt(count / (4.0 * np.pi))) / n,
                                           [0.5, 0.48, 0.51])))
@@ -40,6 +43,17 @@ def test_large_counts(cuda_device, which):
     x, it = s.apply_c_inverse(t, c_rtol=1e-13, c_maxit=2000)
     r = t - s.interp(s.spread(x))
     assert float(r.norm() / t.norm()) < 3e-12
+    if which == "first_launched":   # its own end tests, host-side
+        from paper_2501_15314_gb300 import _lib
+        with pytest.raises(_lib.IBMError) as e:
+            s.apply_c_inverse(t, c_rtol=1e-13, c_maxit=6)
+        assert e.value.status == _lib.IBM_ERR_NOT_CONVERGED
+        x, it = s.apply_c_inverse(0.0 * t)
+        assert it == 0 and float(x.abs().max()) == 0.0
+        t[5] = np.nan
+        with pytest.raises(_lib.IBMError) as e:
+            s.apply_c_inverse(t)
+        assert e.value.status == _lib.IBM_ERR_NAN
     s.close()
 
 
