@@ -259,7 +259,7 @@ ibm_status ibm_apply_schur_opts(ibm_ctx* ctx, const double* v, double* out,
 /* s = C^{-1} t with C = R^T R ([3][n_markers] device vectors, t and s must
  * not alias): conjugate gradients on C, to ||t - C s|| <= c_rtol ||t|| within
  * c_maxit iterations (IBM_ERR_NOT_CONVERGED otherwise, s holds the last
- * iterate).  The first call after ibm_set_markers forms C's rows (about 36
+ * iterate).  The first call after ibm_set_markers forms C's rows (about 58
  * entries per marker and component at spacing h); many or dense markers
  * are multiplied matrix-free (spread to the shell faces, interpolate back).
  * iters may be NULL.  Synchronises. */

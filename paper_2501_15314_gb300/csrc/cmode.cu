@@ -14,14 +14,14 @@
 // separated by grid-wide barriers, which carry the partial sums of the two dot
 // products with them.  Three forms:
 //   rows: C's rows are formed once per marker set (the overlaps of the markers'
-//     supports, about 36 per marker at spacing h) and kept until the markers
+//     supports, about 58 per marker at spacing h) and kept until the markers
 //     change; an iteration is one product and two barriers.  The vectors'
 //     own values stay in registers.
 //   spread: C v = R^T (R v) through the shell faces (written, not accumulated,
 //     so the rest of the face scratch is never read); four barriers.  For more
-//     markers than the grid's registers hold, or rows longer than kRowMax on
-//     average (markers much denser than h), where the rows cost more memory
-//     and time than the spread's 64 + 27 weights.
+//     markers than the grid's registers hold, or rows longer on average than
+//     kRowMax (markers denser than h), which take longer than the spread's
+//     64 + 27 weights.
 //   launched: the spread form's phases as kernels of full grids, nine per
 //     iteration, the residual read by the host every four.  For more than
 //     kOneLaunchMax markers, where an iteration waits on memory for longer than
@@ -51,7 +51,13 @@ constexpr int kCheck = 4;      // the residual is tested every four iterations
 constexpr int kRowLanes = 4;   // lanes per row and component
 constexpr int kRowUnits = 32 / kRowLanes;   // rows a warp takes at once
 constexpr int kRowHeld = 4;    // rows a lane group holds in registers
-constexpr int kRowMax = 256;   // longest average row of the rows form
+// Longest average row of the rows form, where each lane group has one row and
+// where it has several.  Measured, us per iteration rows / spread: 500 markers
+// 14.5 / 18.6 with rows of 98, 19.7 / 19.5 with 148; 4000 markers 17.5 / 20.8 and
+// 22.3 / 21.5; 8000 (two rows a group) 29.9 / 29.9 with 60, 31.9 / 24.8 with 98;
+// 25000 (four) 37.8 / 46.1 with 58, 62 / 44 with 98, 161 / 48 with 215.
+constexpr int kRowMax = 112;
+constexpr int kRowMaxMany = 64;
 // polls before a barrier gives up (about a second; a barrier takes microseconds)
 constexpr int kSpinLimit = 1 << 20;
 
@@ -533,8 +539,10 @@ ibm_status form_rows(ibm_ctx* c, CgArgs& a, int sms, bool& rows) {
   rows = false;
   if (3 * mk.n > (int64_t)sms * kCgWarps * kRowUnits * kRowHeld) return IBM_OK;
   if (mk.n > c->m) return IBM_OK;   // the scan's scratch is sized by the cells
-  // segments much longer than at the marker spacings the method works with
-  if (mk.n_entries > (int64_t)kRowMax * mk.n_shell) return IBM_OK;
+  const int64_t row_max =
+      3 * mk.n <= (int64_t)sms * kCgWarps * kRowUnits ? kRowMax : kRowMaxMany;
+  // a marker's row holds all markers of each of its cells
+  if (mk.n_entries > row_max * mk.n_shell) return IBM_OK;
   cudaStream_t str = c->stream;
   const int blocks = div_up(32 * mk.n, TPB);
   if (!mk.c_formed) {
@@ -550,7 +558,7 @@ ibm_status form_rows(ibm_ctx* c, CgArgs& a, int sms, bool& rows) {
     IBM_CUDA(c, cudaStreamSynchronize(str));
     int64_t entries = c->host_flag[0];
     mk.c_n = 0;
-    if (entries > (int64_t)kRowMax * mk.n) entries = 0;   // too long: the spread form
+    if (entries > row_max * mk.n) entries = 0;   // too long: the spread form
     if (entries > mk.c_val_cap) {
       cudaFree(mk.c_val);
       mk.c_val_cap = 0;

@@ -57,25 +57,28 @@ def test_large_counts(cuda_device, which):
     s.close()
 
 
-def _dense(which):
-    """Markers on a 32^3 grid."""
+def _dense(which, n=32):
+    """Markers on an n^3 grid."""
     rng = np.random.default_rng(8)
-    h = 1.0 / 32
+    h = 1.0 / n
     cell = np.array([[0.5], [0.47], [0.44]])
     if which == "cell_of_100":       # rows form; 100 entries in the shared cells
         return np.concatenate([cell + rng.uniform(0.0, 0.9 * h, (3, 100)),
                                wl.fibonacci_sphere(700, 0.25, [0.5, 0.5, 0.5])], axis=1)
     if which == "entries":           # 600 entries a cell
         return cell + rng.uniform(0.0, 0.9 * h, (3, 600))
+    if which == "rows_of_two":       # 90 in a row, too long for two rows a lane group
+        return 10 * h + rng.uniform(0.0, 28 * h, (3, 7000))
     # "rows": one and a half markers a cell, about 360 in a row
     return 8 * h + rng.uniform(0.0, 16 * h, (3, 6144))
 
 
-@pytest.mark.parametrize("which", ["cell_of_100", "entries", "rows"])
-def test_dense_markers(cuda_device, which):
+@pytest.mark.parametrize("which,n", [("cell_of_100", 32), ("entries", 32), ("rows", 32),
+                                     ("rows_of_two", 64)])
+def test_dense_markers(cuda_device, which, n):
     from paper_2501_15314_gb300.api import IBMSolver
-    X = _dense(which)
-    s = IBMSolver(32)
+    X = _dense(which, n)
+    s = IBMSolver(n)
     s.set_markers(dev(X))
     y = dev(np.random.default_rng(9).standard_normal(X.size))
     t = s.interp(s.spread(y))
