@@ -49,7 +49,7 @@ void cheb_weights(int p, double* w) {
 // in four additions (the pair x(i-1,k) + x(i,k-1) serves the cells (i,k) and
 // (i-1,k-1)), the smoothing step in three operations on top of it, the
 // restriction from the differences across the faces of the coarse cell (the
-// differences inside it cancel; 4 operations per fine cell), the prolongation
+// differences inside it cancel; 4 1/4 operations per fine cell), the prolongation
 // separably with its powers of 1/4 in one factor (3 1/4).  Per V-cycle at the
 // finest level about 30 FP64 operations per cell.  Measured at 192^3 in FP64
 // (us per launch, in brackets one cell's plain sums and quotients in marches
@@ -266,11 +266,18 @@ __global__ void __launch_bounds__(BX * BY) k_first(Dims d, const TB* __restrict_
 // Residual restriction: bcoarse = average over the 8 children of (b - L x);
 // x == nullptr means x = 0.  A thread owns one fine x and the two fine rows of
 // a coarse one, and marches over the coarse planes.  The sum of L x over the
-// children is the sum of the differences across the coarse cell's faces.
+// children is the sum of the differences across the coarse cell's faces; it is
+// formed, and taken from b, for each of the two fine planes, whose sums are small
+// enough that the rounding error is no larger than cell by cell (measured alone
+// on rough b: 0.95 of that at 48^3, 0.89 at 96^3, on smooth b 0.48 and 0.33; in
+// one sum over both planes 1.45 and 1.13).  Three blocks per SM (80 registers): the
+// V-cycle at 64^3 takes 78.3 us, with four and their spills 79.8.
 template <typename T>
-__global__ void __launch_bounds__(BX * BY, 4) k_restrict(Dims d, Dims dc, const T* __restrict__ x,
-                                                      const T* __restrict__ b,
-                                                      T* __restrict__ bcoarse, T inv_h2, int zcc) {
+__global__ void __launch_bounds__(BX * BY, 3) k_restrict(Dims d, Dims dc,
+                                                         const T* __restrict__ x,
+                                                         const T* __restrict__ b,
+                                                         T* __restrict__ bcoarse, T inv_h2,
+                                                         int zcc) {
   pdl_wait();
   pdl_trigger();
   const int lane = threadIdx.x;
@@ -296,9 +303,11 @@ __global__ void __launch_bounds__(BX * BY, 4) k_restrict(Dims d, Dims dc, const 
     sm = K0 > 0 ? __ldg(x + c - sz) + __ldg(x + c - sz + sy) : s0;
   }
   for (int K = K0; K < K1; ++K, c += 2 * sz) {
-    T r = 0, t = 0;
-    if (act)
-      r = (__ldg(b + c) + __ldg(b + c + sy)) + (__ldg(b + c + sz) + __ldg(b + c + sz + sy));
+    T r0 = 0, r1 = 0;   // the two planes' sums over the rows
+    if (act) {
+      r0 = __ldg(b + c) + __ldg(b + c + sy);
+      r1 = __ldg(b + c + sz) + __ldg(b + c + sz + sy);
+    }
     if (x) {
       T e0 = 0, e1 = 0, n0 = 0, n1 = 0;
       T m0 = a0, m1 = 0, p0 = a1, p1 = 0;   // y-neighbours of the two planes
@@ -321,21 +330,23 @@ __global__ void __launch_bounds__(BX * BY, 4) k_restrict(Dims d, Dims dc, const 
         }
       }
       const T s1 = e0 + e1, s2 = n0 + n1;
-      const T cc = s0 + s1;
-      T oc = __shfl_sync(0xffffffffu, cc, src & 31);
-      if (lane == 0 || lane == 31)
-        oc = edge ? (__ldg(x + c + eo) + __ldg(x + c + sy + eo)) +
-                        (__ldg(x + c + sz + eo) + __ldg(x + c + sz + sy + eo))
-                  : (T)0;
-      if (wallx) oc = cc;
-      t = fma((T)3, cc,
-              -((oc + ((m0 + p0) + (m1 + p1))) + (sm + (K < dc.nz - 1 ? s2 : s1))));
+      T o0 = __shfl_sync(0xffffffffu, s0, src & 31), o1 = __shfl_sync(0xffffffffu, s1, src & 31);
+      if (lane == 0 || lane == 31) {
+        o0 = edge ? __ldg(x + c + eo) + __ldg(x + c + sy + eo) : (T)0;
+        o1 = edge ? __ldg(x + c + sz + eo) + __ldg(x + c + sz + sy + eo) : (T)0;
+      }
+      if (wallx) {
+        o0 = s0;
+        o1 = s1;
+      }
+      r0 = fma(-inv_h2, fma((T)3, s0, -((o0 + (m0 + p0)) + sm)), r0);
+      r1 = fma(-inv_h2, fma((T)3, s1, -((o1 + (m1 + p1)) + (K < dc.nz - 1 ? s2 : s1))), r1);
       sm = s1;
       s0 = s2;
       a0 = n0;
       a1 = n1;
     }
-    r = fma(-inv_h2, t, r);
+    T r = r0 + r1;
     r += __shfl_xor_sync(0xffffffffu, r, 1);
     if (act && !(lane & 1)) bcoarse[((int64_t)K * dc.ny + J) * dc.nx + (i >> 1)] = r * (T)0.125;
   }
