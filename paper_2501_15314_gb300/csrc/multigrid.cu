@@ -54,7 +54,7 @@ void cheb_weights(int p, double* w) {
 // finest level about 30 FP64 operations per cell.  Measured at 192^3 in FP64
 // (us per launch, in brackets one cell's plain sums and quotients in marches
 // of 16 planes): k_first 115 (513), k_sweep 112 (249; 94 at 600 G/s),
-// k_restrict 77 (133), k_prolong 61 (174), the V-cycle 612 (2230).
+// k_restrict 78 (133), k_prolong 61 (174), the V-cycle 614 (2230).
 // The levels below 64^3 are bound by latency: one plane per thread (zm_planes)
 // and programmatic dependent launch.
 //
@@ -268,10 +268,11 @@ __global__ void __launch_bounds__(BX * BY) k_first(Dims d, const TB* __restrict_
 // a coarse one, and marches over the coarse planes.  The sum of L x over the
 // children is the sum of the differences across the coarse cell's faces; it is
 // formed, and taken from b, for each of the two fine planes, whose sums are small
-// enough that the rounding error is no larger than cell by cell (measured alone
-// on rough b: 0.95 of that at 48^3, 0.89 at 96^3, on smooth b 0.48 and 0.33; in
-// one sum over both planes 1.45 and 1.13).  Three blocks per SM (80 registers): the
-// V-cycle at 64^3 takes 78.3 us, with four and their spills 79.8.
+// enough that the rounding error is that of the residuals formed cell by cell
+// (this stage's error alone, relative to theirs: 1.05 at 48^3 and 0.96 at 96^3 on
+// rough b, 0.55 and 0.41 on smooth b; in one sum over both planes 1.32 and 1.17 on
+// rough b).  Three blocks per SM (80 registers): the V-cycle at 64^3 takes
+// 78.3 us, with four and their spills 79.8.
 template <typename T>
 __global__ void __launch_bounds__(BX * BY, 3) k_restrict(Dims d, Dims dc,
                                                          const T* __restrict__ x,
@@ -870,6 +871,9 @@ __global__ void __launch_bounds__(32 * VY) k_prolong_v4(Dims d, Dims dc,
 // saves more than the repeated interpolation costs: 8.1 us against 4.3 + 5.1 at
 // 64^3, 5.2 against 3.8 + 4.6 at 32^3; at 128^3 it is 21 against 8.2 + 7.0, at
 // 256^3 (in marches of four planes, 128 registers) 108 against 36 + 27.
+// Between the two the line hardly matters: FP32 V-cycles with the finest level
+// fused / not fused, us: 32^3 26.4 / 27.6, 64^3 44.0 / 46.2, 80^3 54.3 / 55.1, 96^3
+// 62.5 / 62.4, 112 x 80 x 96 61.2 / 61.1, 128^3 80.5 / 79.6.
 constexpr int64_t kFuseCells = 300000;
 
 template <typename TO>
