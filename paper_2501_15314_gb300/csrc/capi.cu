@@ -294,19 +294,22 @@ ibm_status helmholtz_solve(ibm_ctx* c, const double* rhs, double* u, const ibm_s
     }
     *relres = rn / base;
     if (*relres <= o->helm_rtol || rn == 0.0 || it >= o->helm_maxit) break;
-    // Reduction wanted from this correction (with a 3x margin), FP32-limited.
-    // After n half-steps one colour holds step n of the full iteration and the
-    // other step n - 1; the residual is at most (1 - rho tau) / (1 - rho) times
+    // Reduction needed, by this correction with a 3x margin, FP32-limited.  After
+    // n half-steps one colour holds step n of the full iteration and the other
+    // step n - 1; the residual is at most gain = (1 - rho tau) / (1 - rho) times
     // 1 / T_{n-1}(1 / rho) of the first, tau the iteration's decay per step.
-    // A correction at the FP32 limit, with more to follow, has no target to
-    // meet exactly: it takes the step count of 1 / T_n.
-    const double want = o->helm_rtol / *relres / 3.0;
+    // Where a correction cannot reach the target and the ones still allowed leave
+    // room, it takes the n of 1 / T_n: the next one makes up for the rest.
+    const double need = o->helm_rtol / *relres;
     const double decay = std::acosh(1.0 / rho);
     const double tau = rho / (1.0 + std::sqrt(1.0 - rho * rho));
     const double gain = (1.0 - rho * tau) / (1.0 - rho);
-    int K = want < 1e-6 ? (int)std::ceil(std::acosh(1e6) / decay)
-                        : 1 + (int)std::ceil(std::acosh(std::max(gain / want, 1.0)) / decay);
-    K = K < 3 ? 3 : (K > 120 ? 120 : K);
+    const bool more =
+        need < 1e-6 && std::pow(1e-6 * gain * std::exp(decay), o->helm_maxit - it) <= need;
+    const double steps =
+        more ? std::ceil(std::acosh(1e6) / decay)
+             : 1.0 + std::ceil(std::acosh(std::max(gain / std::max(need / 3.0, 1e-6), 1.0)) / decay);
+    const int K = steps < 3.0 ? 3 : (steps < 120.0 ? (int)steps : 120);
     // half-step 1 (colour 0 from zero) came with the residual
     double omega = 2.0;
     for (int q = 2; q <= K; ++q) {
