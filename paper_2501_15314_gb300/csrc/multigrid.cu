@@ -54,7 +54,7 @@ void cheb_weights(int p, double* w) {
 // finest level about 30 FP64 operations per cell.  Measured at 192^3 in FP64
 // (us per launch, in brackets one cell's plain sums and quotients in marches
 // of 16 planes): k_first 115 (513), k_sweep 112 (249; 94 at 600 G/s),
-// k_restrict 78 (133), k_prolong 61 (174), the V-cycle 614 (2230).
+// k_restrict 78 (133), k_prolong 61 (174), the V-cycle 607 (2230).
 // The levels below 64^3 are bound by latency: one plane per thread (zm_planes)
 // and programmatic dependent launch.
 //
@@ -271,8 +271,10 @@ __global__ void __launch_bounds__(BX * BY) k_first(Dims d, const TB* __restrict_
 // enough that the rounding error is that of the residuals formed cell by cell
 // (this stage's error alone, relative to theirs: 1.05 at 48^3 and 0.96 at 96^3 on
 // rough b, 0.55 and 0.41 on smooth b; in one sum over both planes 1.32 and 1.17 on
-// rough b).  Three blocks per SM (80 registers): the V-cycle at 64^3 takes
-// 78.3 us, with four and their spills 79.8.
+// rough b).  Three blocks per SM (80 registers; with four and their spills the
+// V-cycle at 64^3 took 79.8 us instead of 78.3), the values past the warp's edge
+// loaded with the others rather than after the shuffles: 64^3 76.5 -> 74.8 us,
+// 192^3 612.9 -> 606.6.
 template <typename T>
 __global__ void __launch_bounds__(BX * BY, 3) k_restrict(Dims d, Dims dc,
                                                          const T* __restrict__ x,
@@ -312,6 +314,13 @@ __global__ void __launch_bounds__(BX * BY, 3) k_restrict(Dims d, Dims dc,
     if (x) {
       T e0 = 0, e1 = 0, n0 = 0, n1 = 0;
       T m0 = a0, m1 = 0, p0 = a1, p1 = 0;   // y-neighbours of the two planes
+      T g0 = 0, g1 = 0, h0 = 0, h1 = 0;     // x-neighbours past the warp's edge
+      if (edge) {
+        g0 = __ldg(x + c + eo);
+        g1 = __ldg(x + c + sy + eo);
+        h0 = __ldg(x + c + sz + eo);
+        h1 = __ldg(x + c + sz + sy + eo);
+      }
       if (act) {
         e0 = __ldg(x + c + sz);
         e1 = __ldg(x + c + sz + sy);
@@ -332,9 +341,9 @@ __global__ void __launch_bounds__(BX * BY, 3) k_restrict(Dims d, Dims dc,
       }
       const T s1 = e0 + e1, s2 = n0 + n1;
       T o0 = __shfl_sync(0xffffffffu, s0, src & 31), o1 = __shfl_sync(0xffffffffu, s1, src & 31);
-      if (lane == 0 || lane == 31) {
-        o0 = edge ? __ldg(x + c + eo) + __ldg(x + c + sy + eo) : (T)0;
-        o1 = edge ? __ldg(x + c + sz + eo) + __ldg(x + c + sz + sy + eo) : (T)0;
+      if (edge) {
+        o0 = g0 + g1;
+        o1 = h0 + h1;
       }
       if (wallx) {
         o0 = s0;
